@@ -2,6 +2,7 @@
 // (kernels and launch shapes in k_rates.cuh).  The sources' variants are compiled in
 // k_rates_rhs.cu, a translation unit of their own, so the two halves build in parallel.
 #include "k_rates.cuh"
+#include "k_rates_fx.cuh"
 
 namespace nk {
 
@@ -17,6 +18,10 @@ cudaError_t launch_rates(const DevMech& m, int64_t n, int64_t ld, const double* 
     if (rhs) return launch_rates_rhs(m, n, ld, T, p, Y, dlnA, omega, hrr, precision, s);
     if (precision == NK_MIXED) return launch_form<kMixed, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
     if (precision == NK_FP64_NATIVE) return launch_form<kNative, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+    if (m.fx_ok) {
+        const cudaError_t e = launch_rates_fx<false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+        return e != cudaSuccess ? e : launch_marked<false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+    }
     return launch_form<kDF, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
 }
 

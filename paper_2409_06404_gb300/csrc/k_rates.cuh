@@ -15,7 +15,8 @@
 // Three arithmetic forms (template PREC):
 //  kNative (NK_FP64_NATIVE): every operation in double (exp/log from nk_math.cuh), with the
 //    per-species g_k/RT in shared memory.
-//  kDF (NK_FP64): the exponent chains -- the reaction's Gibbs sum (from its thermo groups),
+//  kDF (NK_FP64 for the points and mechanisms outside the fixed-point form, k_rates_fx.cuh, which
+//    takes all others): the exponent chains -- the reaction's Gibbs sum (from its thermo groups),
 //    ln k_f, ln K_c, the Troe falloff -- in double-float pairs on the FP32 pipe (nk_df.cuh),
 //    each exponential returned as a double with one FP64 add; the concentrations enter the
 //    rate terms' exponents as pair logarithms (their signs beside them), and the rate terms,
@@ -30,6 +31,7 @@
 #include <utility>
 #include <vector>
 
+#include "nk_fxpt.cuh"
 #include "nk_rxn.cuh"
 
 namespace nk {
@@ -357,7 +359,7 @@ __host__ __device__ constexpr int shared_rows() {
 //
 // RHS: write the implicit-stage sources instead: omega -> W_k omega_k / rho, hrr -> hrr/(rho c_p).
 //
-// PASS (kDF and kMixed): 0 takes the blocks without a negative concentration and skips the
+// PASS 2 (kDF): as 1 for the points whose hrr holds kFxSkip, whatever their state.  PASS (kDF and kMixed): 0 takes the blocks without a negative concentration and skips the
 // others, 1 takes only those, with the concentrations' signs in a byte row after the omega_k row
 // (rates_smem_signs); so the common pass carries no sign work.  The second pass leaves at once
 // where no mass fraction of the block is negative.  The native form has one pass (0) over every
@@ -381,8 +383,13 @@ __global__ void __launch_bounds__(BLK * NP, (PREC != kNative ? 768 : 640) / (BLK
     const int slot = threadIdx.x % BLK, part = threadIdx.x / BLK;
     const int64_t i0 = (int64_t)blockIdx.x * BLK + slot;
     if (NP == 1 && i0 >= n) return;              // (NP = 1 has no block barrier below)
-    const bool live = i0 < n;
+    bool live = i0 < n;
     const int64_t i = live ? i0 : n - 1;         // idle slots of the last block recompute point n-1
+    if constexpr (PASS == 2) {
+        const bool marked = __double_as_longlong(hrr[i]) == (long long)kFxSkip;
+        if (!(NP > 1 ? __syncthreads_or(marked) != 0 : __any_sync(__activemask(), marked))) return;
+        live &= marked;
+    }
     if constexpr (PREC != kNative && PASS == 1) {
         // no negative mass fraction and positive T and p in the block (its warp for NP = 1): no
         // concentration is negative (rho > 0), the logarithmic pass took it; anything else goes
@@ -396,7 +403,7 @@ __global__ void __launch_bounds__(BLK * NP, (PREC != kNative ? 768 : 640) / (BLK
     double* sG = smem + kMathTabDoubles + (size_t)K * BLK + slot;     // g_k / RT (native form)
     double* sW0 = smem + kMathTabDoubles + (size_t)shared_rows<PREC>() * K * BLK + slot;
     double* sW = sW0;                                                  // omega_k
-    constexpr bool SG = PREC != kNative && PASS == 1;
+    constexpr bool SG = PREC != kNative && PASS >= 1;
     uint8_t* sg = reinterpret_cast<uint8_t*>(sW0 - slot + (size_t)K * BLK) + slot;   // (SG) sign of C_k
 
     Pt P;
@@ -440,7 +447,7 @@ __global__ void __launch_bounds__(BLK * NP, (PREC != kNative ? 768 : 640) / (BLK
     } else if constexpr (PREC != kNative) {
         vote = __any_sync(__activemask(), neg);
     }
-    if constexpr (PREC != kNative) {
+    if constexpr (PREC != kNative && PASS < 2) {
         if (PASS == 0 ? vote : !vote) return;     // the other pass takes this block
     }
 
@@ -548,6 +555,20 @@ cudaError_t launch_idx(int idx, std::integer_sequence<int, S...>, const DevMech&
     return e;
 }
 
+
+// The points that the fixed-point kernel (k_rates_fx.cuh) left marked in hrr, in the kDF form with
+// signs (any state).
+template <bool RHS>
+cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
+                          const double* dlnA, double* omega, double* hrr, cudaStream_t st) {
+    const Shape sh{32, m.K >= 8 ? 4 : 1};
+    const size_t smem = rates_smem<kDF>(m.K, sh) + rates_smem_signs(m.K, sh);
+    auto kern = sh.np == 4 ? rates_kernel<32, 4, kDF, RHS, 2> : rates_kernel<32, 1, kDF, RHS, 2>;
+    const cudaError_t e = ensure_smem((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((n + 31) / 32), 32 * sh.np, smem, st>>>(m, n, ld, T, p, Y, dlnA, omega, hrr);
+    return cudaGetLastError();
+}
 
 // The shape with the most resident warps per SM (CUDA's occupancy calculator: shared memory,
 // registers, threads), fewer parts on ties.  Cached per

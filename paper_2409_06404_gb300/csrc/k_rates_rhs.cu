@@ -1,6 +1,7 @@
 // The implicit-stage sources' variants of the rates kernel (k_rates.cuh), compiled apart from the
 // rates' variants (k_rates.cu) so the two build in parallel.
 #include "k_rates.cuh"
+#include "k_rates_fx.cuh"
 
 namespace nk {
 
@@ -9,6 +10,10 @@ cudaError_t launch_rates_rhs(const DevMech& m, int64_t n, int64_t ld, const doub
                              cudaStream_t s) {
     if (precision == NK_MIXED) return launch_form<kMixed, true>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
     if (precision == NK_FP64_NATIVE) return launch_form<kNative, true>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+    if (m.fx_ok) {
+        const cudaError_t e = launch_rates_fx<true>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+        return e != cudaSuccess ? e : launch_marked<true>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+    }
     return launch_form<kDF, true>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
 }
 

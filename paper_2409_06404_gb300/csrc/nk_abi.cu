@@ -10,6 +10,7 @@
 #include <map>
 #include <vector>
 
+#include "fx_tables.h"
 #include "nk_internal.cuh"
 
 namespace {
@@ -515,6 +516,8 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
             for (int j = 0; j < 5; ++j)
                 f_cp[((size_t)k * 2 + range) * 8 + j] = (float)nasa[((size_t)k * 2 + range) * nk::kNasaStride + j];
 
+    const nk::FxTables fxt = nk::build_fx_tables(K, rxn, troe, eff_sp, eff_m1, nasa, d->W, d->T_mid);
+
     // ---- one device block for everything
     Layout L;
     const size_t o_W = L.add(K * 8), o_invW = L.add(K * 8), o_Tmid = L.add(K * 8), o_nasa = L.add(nasa.size() * 8),
@@ -540,7 +543,12 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
                  o_rv4 = L.add(rsched[3].size() * 4 + 16), o_mp2 = L.add(mt_ptr[0].size() * 4 + 16),
                  o_mp4 = L.add(mt_ptr[1].size() * 4 + 16), o_ms2 = L.add(mt_slot[0].size() * 4 + 16),
                  o_ms4 = L.add(mt_slot[1].size() * 4 + 16), o_me2 = L.add(mt_eps[0].size() * 8 + 16),
-                 o_me4 = L.add(mt_eps[1].size() * 8 + 16);
+                 o_me4 = L.add(mt_eps[1].size() * 8 + 16), o_xtab = L.add(fxt.tab.size() * 4),
+                 o_xr = L.add(fxt.chunks.size() + 16),
+                 o_xx = L.add(fxt.extra.size() * sizeof(nk::FxExtra) + 16),
+                 o_xt = L.add(fxt.troe.size() * sizeof(nk::FxTroe) + 16),
+                 o_xs = L.add(fxt.sp.size() * sizeof(nk::FxSpecies)),
+                 o_xe = L.add(fxt.eff.size() * sizeof(nk::FxEff) + 16);
     std::vector<unsigned char> host(L.bytes, 0);
     auto put = [&](size_t off, const void* src, size_t n) {
         if (n) std::memcpy(host.data() + off, src, n);
@@ -601,6 +609,12 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
     put(o_fcp, f_cp.data(), f_cp.size() * 4);
     put(o_lcw, lc_w.data(), lc_w.size() * 8);
     put(o_dfe, df_effm1.data(), df_effm1.size() * 8);
+    put(o_xtab, fxt.tab.data(), fxt.tab.size() * 4);
+    put(o_xr, fxt.chunks.data(), fxt.chunks.size());
+    put(o_xx, fxt.extra.data(), fxt.extra.size() * sizeof(nk::FxExtra));
+    put(o_xt, fxt.troe.data(), fxt.troe.size() * sizeof(nk::FxTroe));
+    put(o_xs, fxt.sp.data(), fxt.sp.size() * sizeof(nk::FxSpecies));
+    put(o_xe, fxt.eff.data(), fxt.eff.size() * sizeof(nk::FxEff));
 
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -688,6 +702,22 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
     dm.mt_slot4 = reinterpret_cast<const int32_t*>(b + o_ms4);
     dm.mt_eps2 = reinterpret_cast<const double*>(b + o_me2);
     dm.mt_eps4 = reinterpret_cast<const double*>(b + o_me4);
+    dm.fx_ok = fxt.ok ? 1 : 0;
+    dm.fx_rows = fxt.rows;
+    dm.fx_image = fxt.image;
+    dm.fx_image_parts = fxt.image_parts;
+    dm.fx_image_spec = fxt.image_spec;
+    dm.fx_image_list = fxt.image_list;
+    dm.fx_nchunk = fxt.nchunk;
+    dm.fx_eff_shift = fxt.eff_shift;
+    dm.fx_lmaxw = (int64_t)llroundl((long double)fxt.log2_maxinvW * 281474976710656.0L);
+    dm.fx_lR = (int64_t)llroundl(log2l((long double)nk::kR) * 281474976710656.0L);
+    dm.fx_tab = reinterpret_cast<const uint32_t*>(b + o_xtab);
+    dm.fx_chunks = b + o_xr;
+    dm.fx_extra = reinterpret_cast<const nk::FxExtra*>(b + o_xx);
+    dm.fx_troe = reinterpret_cast<const nk::FxTroe*>(b + o_xt);
+    dm.fx_sp = reinterpret_cast<const nk::FxSpecies*>(b + o_xs);
+    dm.fx_eff = reinterpret_cast<const nk::FxEff*>(b + o_xe);
     dm.mslots2 = mslots[0];
     dm.mslots4 = mslots[1];
     for (int g = 0; g < 4; ++g) {

@@ -94,6 +94,52 @@ struct __align__(16) JacTerm {
     int32_t slot, dst;
 };
 
+// Fixed-point tables (nk_fx.cuh, built by fx_tables.cu): logarithms to base 2 in units of 2^-48.
+// One reaction: ln k_f = lnA + beta lt + Ea v with fx_mul and the point's fractions of log2 T and
+// 1/T; off: byte offsets of its molecules' rows (kFxRow per species slot; a coefficient nu repeats its
+// species), reactants at [0, nr), products at [4, 4 + np); the first two of each side always name
+// a row (the row after the last species holds zeros).  info = nr | np << 4 | kind << 8 |
+// index of the FxExtra record (third-body and Troe) << 16.
+constexpr int kFxRow = 512;       // a species' row: log2 C_k and mu_k of 32 points
+struct __align__(16) FxRxn {
+    int64_t lnA, beta, Ea;
+    int32_t info, orig;
+    uint32_t off[8];
+};
+static_assert(sizeof(FxRxn) == 64, "fixed-point reaction record");
+struct __align__(16) FxExtra {
+    int32_t eff0, eff1, aux, pad;  // third-body efficiencies [eff0, eff1), Troe record or -1
+};
+// Chunks: up to kFxChunk reactions whose rates of progress are staged together.  A chunk's image
+// (fx_image bytes, a multiple of 16) holds its reaction records in schedule order (part by part,
+// balanced by cost), then at image_parts the first record of each part (NP + 1 bytes), at
+// image_spec one word per species slot (start in the list << 16 | rows to add << 8 | rows to
+// subtract) and at image_list the rows as 16-bit byte offsets (256 per row).
+constexpr int kFxChunk = 48;
+// One Troe reaction: its low-pressure limit as FxRxn's, and F_cent's terms: log2(1 - a),
+// -log2(e)/T3 times T, log2 a, -log2(e)/T1 times T and -log2(e) T2 times 1/T (flags: 1 the terms
+// fit, 2 the last one is there).
+struct __align__(16) FxTroe {
+    int64_t lnA0, beta0, Ea0, l3, x3, l1, x1, x2;
+    int64_t flags, pad;
+};
+// One species, in slot order (slot s belongs to part s % NP; the species are dealt so that the parts
+// sum about equally many rates of progress): its index k, log2(1/W), 1/W relative to the largest (units 2^-62), T_mid, and per range the
+// polynomials in T/4096, log2 T and 1/T of log2(e) g/RT + log2(R T/p0) (c[0..6]: constant, log2 T,
+// T..T^4, 1/T), h/RT (c[8..13]: constant, T..T^4, 1/T) and c_p/R over kFxCpScale (c[7], then
+// T..T^4 in c[14..17]).
+constexpr double kFxCpScale = 8.0;
+struct __align__(16) FxSpecies {
+    int64_t lw, w;
+    double Tmid;
+    int32_t k, pad;
+    int64_t c[2][18];
+};
+struct __align__(16) FxEff {
+    int64_t w;          // (eps - 1)/W relative to the largest 1/W, units 2^(eff_shift - 62)
+    int32_t sp, pad;
+};
+
 constexpr int kTroeDf = 4;       // float4 records per Troe reaction in DevMech::troe_df
 
 // Device view of a loaded mechanism (passed by value to every kernel).
@@ -184,6 +230,16 @@ struct DevMech {
     // (reactants at [0, nr), products at [kMaxSide, kMaxSide + np); nu_first the side's first entry)
     const double* lc_w;           // [R][2 kMaxSide]
     const float2* df_eff_m1;      // efficiencies - 1 as pairs (eff_m1 order)
+    // fixed-point tables of the FP64 reaction kernels (fx_ok: the mechanism fits them)
+    int32_t fx_ok, fx_rows, fx_nchunk, fx_eff_shift;      // fx_rows: the largest chunk's reactions
+    int32_t fx_image, fx_image_parts, fx_image_spec, fx_image_list;
+    int64_t fx_lmaxw, fx_lR;      // log2(largest 1/W), log2(R)
+    const uint32_t* fx_tab;
+    const unsigned char* fx_chunks;   // [fx_nchunk][fx_image]
+    const FxExtra* fx_extra;
+    const FxTroe* fx_troe;
+    const FxSpecies* fx_sp;           // [K] in slot order
+    const FxEff* fx_eff;
 };
 
 // Centre of the re-expanded transport fits (ln T about 1100 K).
@@ -197,6 +253,12 @@ struct JitModule {
     void* lib = nullptr;    // cudaLibrary_t
     void* kern = nullptr;   // cudaKernel_t
 };
+}  // namespace nk
+
+namespace nk {
+constexpr int kFxOwn = 8;          // species per part of the fixed-point kernels, at most
+// Parts (warps) per point for K species.
+inline int fx_parts(int K) { return K <= 4 * kFxOwn ? 4 : K <= 8 * kFxOwn ? 8 : K <= 16 * kFxOwn ? 16 : 32; }
 }  // namespace nk
 
 // The opaque handle of the public ABI.

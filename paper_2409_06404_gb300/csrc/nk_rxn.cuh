@@ -190,10 +190,11 @@ static __device__ __noinline__ TroeCent troe_cent_edge(const TroeRec* t, double 
     const double Fc = e3 + e1 + e2, FT = e2 * x2 - e3 * x3 - e1 * x1;
     return TroeCent{df_split_cvt(log10(Fc)), df_split_cvt(FT / (Fc * 2.302585092994046))};
 }
-__device__ __forceinline__ TroeCent troe_cent(const DevMech& m, int aux, const TPairs& P, const DfTab& dt) {
-    const float4 t1 = __ldg(m.troe_df + kTroeDf * aux + 1);    // (Ea0/R, 1/T3)
-    const float4 t2 = __ldg(m.troe_df + kTroeDf * aux + 2);    // (1/T1, T2)
-    const float4 t3 = __ldg(m.troe_df + kTroeDf * aux + 3);    // (a, 1 - a)
+__device__ __forceinline__ TroeCent troe_cent(const float4* troe_df, const TroeRec* troe, int aux, const TPairs& P,
+                                              const DfTab& dt) {
+    const float4 t1 = __ldg(troe_df + kTroeDf * aux + 1);      // (Ea0/R, 1/T3)
+    const float4 t2 = __ldg(troe_df + kTroeDf * aux + 2);      // (1/T1, T2)
+    const float4 t3 = __ldg(troe_df + kTroeDf * aux + 3);      // (a, 1 - a)
     const dfl x3 = df_mul(P.Td, dfl{t1.z, t1.w}), x1 = df_mul(P.Td, dfl{t2.x, t2.y});
     const dfl e3 = df_mul(dfl{t3.z, t3.w}, exp_df_pair(df_neg(x3), dt.e2));
     const dfl e1 = df_mul(dfl{t3.x, t3.y}, exp_df_pair(df_neg(x1), dt.e2));
@@ -205,8 +206,11 @@ __device__ __forceinline__ TroeCent troe_cent(const DevMech& m, int aux, const T
         Fc = df_add(Fc, e2);
         FT = df_fma(e2, x2, FT);
     }
-    if (!(Fc.h >= 7.888609052210118e-31f)) return troe_cent_edge(m.troe + aux, P.T);
+    if (!(Fc.h >= 7.888609052210118e-31f)) return troe_cent_edge(troe + aux, P.T);
     return TroeCent{df_mul(log_df_pair(Fc, dt.rc, dt.lc), dfc_invln10()), df_mul(df_div(FT, Fc), dfc_invln10())};
+}
+__device__ __forceinline__ TroeCent troe_cent(const DevMech& m, int aux, const TPairs& P, const DfTab& dt) {
+    return troe_cent(m.troe_df, m.troe, aux, P, dt);
 }
 
 // The Troe falloff factor in logarithmic form: for x = ln P_r and L = log10 F_cent,
