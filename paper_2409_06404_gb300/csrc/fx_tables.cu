@@ -39,28 +39,19 @@ const std::vector<uint32_t>& math_tables() {
     return t;
 }
 
-}  // namespace
-
-FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vector<TroeRec>& troe,
-                         const std::vector<int32_t>& eff_sp, const std::vector<double>& eff_m1,
-                         const std::vector<double>& nasa, const double* W, const double* Tmid) {
-    FxTables f;
-    const int R = (int)rxn.size();
+// One kernel family's schedule: species slots and chunk images.
+bool schedule(int set, int K, const std::vector<RxnRec>& rxn, const std::vector<FxRxn>& rec,
+              const std::vector<FxSpecies>& species, FxTables::Set& out) {
+    const int R = (int)rxn.size(), NP = fx_parts(K, set);
+    FxSet& f = out.s;
     bool ok = true;
-    auto put = [&](long double v) {
-        if (!(fabsl(v) < kLimit)) {
-            ok = false;
-            return (int64_t)0;
-        }
-        return fx(v);
-    };
-
-    f.tab = math_tables();
+    f.np = NP;
+    f.row = set == 0 ? kFxRow : kFxDRow;
+    if (NP == 0) return true;              // (the family does not take this mechanism)
 
     // species slots: by decreasing number of molecules over all reactions, dealt to the parts with
     // the fewest so far that still have a place
-    const int NP = fx_parts(K);
-    std::vector<int> slot(K), spec(K);
+    std::vector<int> slot(K);
     {
         std::vector<int> count(K, 0), by(K);
         for (const RxnRec& r : rxn)
@@ -69,136 +60,21 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
         for (int k = 0; k < K; ++k) by[k] = k;
         std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return count[a] > count[b]; });
         std::vector<int> load(NP, 0), used(NP, 0);
+        out.sp.resize(K);
         for (int k : by) {
             int b = -1;
             for (int q = 0; q < NP; ++q)
                 if (q + NP * used[q] < K && (b < 0 || load[q] < load[b])) b = q;
             slot[k] = b + NP * used[b]++;
-            spec[slot[k]] = k;
+            out.sp[slot[k]] = species[k];
             load[b] += count[k];
-        }
-    }
-
-    // species
-    long double maxInv = 0.0L;
-    for (int k = 0; k < K; ++k) maxInv = std::max(maxInv, 1.0L / (long double)W[k]);
-    f.log2_maxinvW = (double)log2l(maxInv);
-    f.sp.resize(K);
-    const long double s = 8192.0L;        // fx_mul halves: T/4096 enters as T/8192, 128/T as 64/T, log2(T)/16 as log2(T)/32
-    const long double l2RP0 = log2l((long double)kR / (long double)kP0);
-    for (int k = 0; k < K; ++k) {
-        FxSpecies& x = f.sp[slot[k]];
-        std::memset(&x, 0, sizeof x);
-        x.k = k;
-        x.lw = put(log2l(1.0L / (long double)W[k]));
-        x.w = (int64_t)llroundl(1.0L / (long double)W[k] / maxInv * 4611686018427387904.0L);   // 2^62
-        x.Tmid = Tmid[k];
-        for (int r = 0; r < 2; ++r) {
-            const double* a = nasa.data() + ((size_t)k * 2 + r) * kNasaStride;
-            int64_t* c = x.c[r];
-            c[0] = put(kL2E * ((long double)a[0] - a[6]) + l2RP0) + 4;       // (+4: fx_mul cuts)
-            c[1] = put(32.0L * (1.0L - (long double)a[0]));
-            c[2] = put(-kL2E * a[1] / 2.0L * s);
-            c[3] = put(-kL2E * a[2] / 6.0L * s * s);
-            c[4] = put(-kL2E * a[3] / 12.0L * s * s * s);
-            c[5] = put(-kL2E * a[4] / 20.0L * s * s * s * s);
-            c[6] = put(kL2E * a[5] / 64.0L);
-            c[8] = put(a[0]);
-            c[9] = put((long double)a[1] / 2.0L * s);
-            c[10] = put((long double)a[2] / 3.0L * s * s);
-            c[11] = put((long double)a[3] / 4.0L * s * s * s);
-            c[12] = put((long double)a[4] / 5.0L * s * s * s * s);
-            c[13] = put((long double)a[5] / 64.0L);
-            c[14] = put((long double)a[1] * s / kFxCpScale);
-            c[15] = put((long double)a[2] * s * s / kFxCpScale);
-            c[16] = put((long double)a[3] * s * s * s / kFxCpScale);
-            c[17] = put((long double)a[4] * s * s * s * s / kFxCpScale);
-            c[7] = put((long double)a[0] / kFxCpScale);
-        }
-    }
-
-    // reactions: flattened molecules (a coefficient nu repeats its species nu times)
-    std::vector<FxRxn> rec(R);
-    for (int q = 0; q < R; ++q) {
-        const RxnRec& r = rxn[q];
-        FxRxn& x = rec[q];
-        std::memset(&x, 0, sizeof x);
-        x.lnA = put(kL2E * r.lnA) + 2;    // (fx_mul cuts about 1.25 units)
-        x.beta = put(32.0L * r.beta);
-        x.Ea = put(-kL2E * r.EaR / 64.0L);
-        x.orig = r.orig;
-        int cnt[2] = {0, 0};
-        for (int e = 0; e < 8; ++e) x.off[e] = (uint32_t)K * kFxRow;
-        for (int side = 0; side < 2; ++side) {
-            const int b = side * kMaxSide, ne = side ? r.np : r.nr;
-            for (int e = 0; e < ne; ++e)
-                for (int j = 0; j < r.nu[b + e]; ++j) {
-                    if (cnt[side] == kMaxSide) {
-                        ok = false;       // more than four molecules on a side
-                        break;
-                    }
-                    x.off[b + cnt[side]++] = (uint32_t)slot[r.sp[b + e]] * kFxRow;
-                }
-        }
-        x.info = cnt[0] | cnt[1] << 4 | r.type << 8;
-        if (r.type != NK_RXN_ELEMENTARY) {
-            x.info |= (int32_t)f.extra.size() << 16;
-            f.extra.push_back(FxExtra{r.eff0, r.eff1, r.aux, 0});
-        }
-    }
-    f.troe.resize(troe.size());
-    for (size_t j = 0; j < troe.size(); ++j) {
-        f.troe[j].lnA0 = put(kL2E * troe[j].lnA0) + 2;
-        f.troe[j].beta0 = put(32.0L * troe[j].beta0);
-        f.troe[j].Ea0 = put(-kL2E * troe[j].Ea0R / 64.0L);
-        f.troe[j].l3 = put(troe[j].a < 1.0 ? log2l(1.0L - (long double)troe[j].a) : 0.0L);
-        f.troe[j].l1 = put(troe[j].a > 0.0 ? log2l((long double)troe[j].a) : 0.0L);
-        f.troe[j].x3 = -kL2E * 8192.0L * troe[j].invT3 > -kLimit ? fx(-kL2E * 8192.0L * troe[j].invT3) : 0;
-        f.troe[j].x1 = -kL2E * 8192.0L * troe[j].invT1 > -kLimit ? fx(-kL2E * 8192.0L * troe[j].invT1) : 0;
-        f.troe[j].x2 = troe[j].hasT2 != 0.0 ? put(-kL2E * troe[j].T2 / 64.0L) : 0;
-        // 0 < a < 1 with exponents in range: F_cent in fixed point
-        f.troe[j].flags = (troe[j].a > 0.0 && troe[j].a < 1.0 && f.troe[j].x3 != 0 && f.troe[j].x1 != 0 ? 1 : 0) |
-                          (troe[j].hasT2 != 0.0 ? 2 : 0);
-    }
-    // (eps - 1)/W relative to the largest 1/W, in units of 2^(eff_shift - 62)
-    long double m = 1.0L;
-    for (size_t j = 0; j < eff_sp.size(); ++j)
-        m = std::max(m, fabsl((long double)eff_m1[j]) / (long double)W[eff_sp[j]] / maxInv);
-    while (ldexpl(1.0L, f.eff_shift) <= m && f.eff_shift < 32) ++f.eff_shift;
-    if (f.eff_shift >= 20) ok = false;
-    f.eff.resize(eff_sp.size());
-    for (size_t j = 0; j < eff_sp.size(); ++j) {
-        f.eff[j].w = ok ? (int64_t)llroundl(ldexpl((long double)eff_m1[j] / (long double)W[eff_sp[j]] / maxInv, 62 - f.eff_shift)) : 0;
-        f.eff[j].sp = eff_sp[j];
-        f.eff[j].pad = 0;
-    }
-
-    // Ranges over the temperature window: rate constants and reaction Gibbs energies together
-    // below kMaxX (so that sums stay inside the format and a zero concentration underflows).
-    const int NT = 64;
-    std::vector<double> G(K);
-    for (int it = 0; it <= NT && ok; ++it) {
-        const double T = kFxTmin * std::pow(kFxTmax / kFxTmin, (double)it / NT), lT = std::log(T), l2e = (double)kL2E;
-        for (int k = 0; k < K; ++k) {
-            const double* a = nasa.data() + ((size_t)k * 2 + (T <= Tmid[k] ? 0 : 1)) * kNasaStride;
-            G[k] = l2e * (a[0] * (1.0 - lT) - T * (a[1] / 2 + T * (a[2] / 6 + T * (a[3] / 12 + T * a[4] / 20))) +
-                          a[5] / T - a[6] + lT) + (double)l2RP0;
-        }
-        for (int q = 0; q < R && ok; ++q) {
-            const RxnRec& r = rxn[q];
-            double g = 0.0;
-            for (int e = 0; e < r.nr; ++e) g -= r.nu[e] * G[r.sp[e]];
-            for (int e = kMaxSide; e < kMaxSide + r.np; ++e) g += r.nu[e] * G[r.sp[e]];
-            const double lk = std::fabs(l2e * (r.lnA + r.beta * lT - r.EaR / T));
-            double l0 = 0.0;
-            if (r.aux >= 0) l0 = std::fabs(l2e * (troe[r.aux].lnA0 + troe[r.aux].beta0 * lT - troe[r.aux].Ea0R / T));
-            ok = lk + std::fabs(g) < kMaxX && l0 < kMaxX;
         }
     }
 
     // Chunks of about equal size with the costlier kinds spread evenly over them; within a chunk
     // the reactions go to the parts by decreasing cost, each to the part with the least so far.
-    f.nchunk = (R + kFxChunk - 1) / kFxChunk;
+    const int chunk = set == 0 ? 48 : 48;
+    f.nchunk = (R + chunk - 1) / chunk;
     std::vector<std::vector<int>> members(f.nchunk);
     for (int kind = 2, next = 0; kind >= 0; --kind)
         for (int q = 0; q < R; ++q)
@@ -240,10 +116,14 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
     f.image_spec = f.image_parts + up(NP + 1);
     f.image_list = f.image_spec + up(4 * K);
     f.image = f.image_list + up(2 * (int)most);
-    f.chunks.assign((size_t)f.nchunk * f.image, 0);
+    out.chunks.assign((size_t)f.nchunk * f.image, 0);
     for (int c = 0; c < f.nchunk; ++c) {
-        unsigned char* im = f.chunks.data() + (size_t)c * f.image;
-        for (size_t i = 0; i < order[c].size(); ++i) std::memcpy(im + i * sizeof(FxRxn), &rec[order[c][i]], sizeof(FxRxn));
+        unsigned char* im = out.chunks.data() + (size_t)c * f.image;
+        for (size_t i = 0; i < order[c].size(); ++i) {
+            FxRxn x = rec[order[c][i]];
+            for (uint32_t& o : x.off) o = (o == (uint32_t)K ? (uint32_t)K : (uint32_t)slot[o]) * (uint32_t)f.row;
+            std::memcpy(im + i * sizeof(FxRxn), &x, sizeof x);
+        }
         std::memcpy(im + f.image_parts, first[c].data(), NP + 1);
         uint32_t at = 0;
         for (int k = 0; k < K; ++k) {
@@ -253,6 +133,191 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
                 for (uint16_t o : *l) std::memcpy(im + f.image_list + 2 * at++, &o, 2);
         }
     }
+    return ok;
+}
+
+}  // namespace
+
+FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vector<TroeRec>& troe,
+                         const std::vector<int32_t>& eff_sp, const std::vector<double>& eff_m1,
+                         const std::vector<double>& nasa, const double* W, const double* Tmid) {
+    FxTables f;
+    const int R = (int)rxn.size();
+    bool ok = true;
+    auto put = [&](long double v) {
+        if (!(fabsl(v) < kLimit)) {
+            ok = false;
+            return (int64_t)0;
+        }
+        return fx(v);
+    };
+
+    f.tab = math_tables();
+
+    // species
+    long double maxInv = 0.0L;
+    for (int k = 0; k < K; ++k) maxInv = std::max(maxInv, 1.0L / (long double)W[k]);
+    f.log2_maxinvW = (double)log2l(maxInv);
+    std::vector<FxSpecies> spec(K);
+    const long double s = 8192.0L;        // fx_mul halves: T/4096 enters as T/8192, 128/T as 64/T, log2(T)/16 as log2(T)/32
+    const long double l2RP0 = log2l((long double)kR / (long double)kP0);
+    for (int k = 0; k < K; ++k) {
+        FxSpecies& x = spec[k];
+        std::memset(&x, 0, sizeof x);
+        x.k = k;
+        x.lw = put(log2l(1.0L / (long double)W[k]));
+        x.w = (int64_t)llroundl(1.0L / (long double)W[k] / maxInv * 4611686018427387904.0L);   // 2^62
+        x.Tmid = Tmid[k];
+        for (int r = 0; r < 2; ++r) {
+            const double* a = nasa.data() + ((size_t)k * 2 + r) * kNasaStride;
+            int64_t* c = x.c[r];
+            c[0] = put(kL2E * ((long double)a[0] - a[6]) + l2RP0) + 4;       // (+4: fx_mul cuts)
+            c[1] = put(32.0L * (1.0L - (long double)a[0]));
+            c[2] = put(-kL2E * a[1] / 2.0L * s);
+            c[3] = put(-kL2E * a[2] / 6.0L * s * s);
+            c[4] = put(-kL2E * a[3] / 12.0L * s * s * s);
+            c[5] = put(-kL2E * a[4] / 20.0L * s * s * s * s);
+            c[6] = put(kL2E * a[5] / 64.0L);
+            c[8] = put(a[0]);
+            c[9] = put((long double)a[1] / 2.0L * s);
+            c[10] = put((long double)a[2] / 3.0L * s * s);
+            c[11] = put((long double)a[3] / 4.0L * s * s * s);
+            c[12] = put((long double)a[4] / 5.0L * s * s * s * s);
+            c[13] = put((long double)a[5] / 64.0L);
+            c[14] = put((long double)a[1] * s / kFxCpScale);
+            c[15] = put((long double)a[2] * s * s / kFxCpScale);
+            c[16] = put((long double)a[3] * s * s * s / kFxCpScale);
+            c[17] = put((long double)a[4] * s * s * s * s / kFxCpScale);
+            c[7] = put((long double)a[0] / kFxCpScale);
+        }
+    }
+
+    // thermo polynomials: per species and quantity the finest unit its coefficients allow
+    {
+        double tm = 0.0;
+        for (int k = 0; k < K; ++k) tm = std::max(tm, Tmid[k]);
+        f.th_lo = 7;
+        while (std::ldexp(1.0 - 1e-9, f.th_lo) <= tm && f.th_lo < 13) ++f.th_lo;
+        bool th = f.th_lo <= 12;
+        f.th.resize(K);
+        for (int k = 0; k < K; ++k) {
+            FxThermo& x = f.th[k];
+            std::memset(&x, 0, sizeof x);
+            x.Tmid = Tmid[k];
+            long double c[2][18], most[3] = {1.0L, 1.0L, 1.0L};
+            for (int r = 0; r < 2; ++r) {
+                const double* a = nasa.data() + ((size_t)k * 2 + r) * kNasaStride;
+                const long double b = ldexpl(1.0L, (r ? 12 : f.th_lo) + 1), R0 = (long double)kR;
+                long double bj = 1.0L;
+                for (int j = 0; j < 5; ++j, bj *= b) {
+                    c[r][j] = R0 * a[j] * bj;
+                    c[r][6 + j] = R0 * a[j] * bj * b / (j + 1);
+                    if (j) c[r][13 + j] = -R0 * a[j] * bj * b / (j * (j + 1));
+                }
+                c[r][5] = c[r][11] = R0 * a[5];
+                c[r][12] = R0 * b * ((long double)a[0] - a[6]);
+                c[r][13] = -R0 * b * a[0] * 32.0L;
+                for (int j = 0; j < 18; ++j) {
+                    long double& m = most[j < 5 ? 0 : j < 11 ? 1 : 2];
+                    m = std::max(m, fabsl(c[r][j]));
+                }
+            }
+            for (int q = 0; q < 3; ++q) {
+                int e = 0;
+                frexpl(most[q], &e);
+                x.sh[q] = 60 - e;          // (sums of up to six terms stay below 2^63)
+                th = th && x.sh[q] > 20;
+            }
+            for (int r = 0; r < 2; ++r)
+                for (int j = 0; j < 18; ++j)
+                    x.c[r][j] = th ? (int64_t)llroundl(ldexpl(c[r][j], x.sh[j < 5 ? 0 : j < 11 ? 1 : 2])) : 0;
+        }
+        if (!th) f.th_lo = 0;
+    }
+
+    // reactions: flattened molecules (a coefficient nu repeats its species nu times)
+    std::vector<FxRxn> rec(R);
+    for (int q = 0; q < R; ++q) {
+        const RxnRec& r = rxn[q];
+        FxRxn& x = rec[q];
+        std::memset(&x, 0, sizeof x);
+        x.lnA = put(kL2E * r.lnA) + 2;    // (fx_mul cuts about 1.25 units)
+        x.beta = put(32.0L * r.beta);
+        x.Ea = put(-kL2E * r.EaR / 64.0L);
+        x.orig = r.orig;
+        int cnt[2] = {0, 0};
+        for (int e = 0; e < 8; ++e) x.off[e] = (uint32_t)K;          // (species; offsets per set below)
+        for (int side = 0; side < 2; ++side) {
+            const int b = side * kMaxSide, ne = side ? r.np : r.nr;
+            for (int e = 0; e < ne; ++e)
+                for (int j = 0; j < r.nu[b + e]; ++j) {
+                    if (cnt[side] == kMaxSide) {
+                        ok = false;       // more than four molecules on a side
+                        break;
+                    }
+                    x.off[b + cnt[side]++] = (uint32_t)r.sp[b + e];
+                }
+        }
+        x.info = cnt[0] | cnt[1] << 4 | r.type << 8;
+        if (r.type != NK_RXN_ELEMENTARY) {
+            x.info |= (int32_t)f.extra.size() << 16;
+            f.extra.push_back(FxExtra{r.eff0, r.eff1, r.aux, 0});
+        }
+    }
+    f.troe.resize(troe.size());
+    for (size_t j = 0; j < troe.size(); ++j) {
+        f.troe[j].lnA0 = put(kL2E * troe[j].lnA0) + 2;
+        f.troe[j].beta0 = put(32.0L * troe[j].beta0);
+        f.troe[j].Ea0 = put(-kL2E * troe[j].Ea0R / 64.0L);
+        f.troe[j].l3 = put(troe[j].a < 1.0 ? log2l(1.0L - (long double)troe[j].a) : 0.0L);
+        f.troe[j].l1 = put(troe[j].a > 0.0 ? log2l((long double)troe[j].a) : 0.0L);
+        f.troe[j].x3 = -kL2E * 8192.0L * troe[j].invT3 > -kLimit ? fx(-kL2E * 8192.0L * troe[j].invT3) : 0;
+        f.troe[j].x1 = -kL2E * 8192.0L * troe[j].invT1 > -kLimit ? fx(-kL2E * 8192.0L * troe[j].invT1) : 0;
+        f.troe[j].x2 = troe[j].hasT2 != 0.0 ? put(-kL2E * troe[j].T2 / 64.0L) : 0;
+        // 0 < a < 1 with exponents in range: F_cent in fixed point
+        f.troe[j].flags = (troe[j].a > 0.0 && troe[j].a < 1.0 && f.troe[j].x3 != 0 && f.troe[j].x1 != 0 ? 1 : 0) |
+                          (troe[j].hasT2 != 0.0 ? 2 : 0);
+    }
+    // (eps - 1)/W relative to the largest 1/W, in units of 2^(eff_shift - 62)
+    long double m = 1.0L;
+    for (size_t j = 0; j < eff_sp.size(); ++j)
+        m = std::max(m, fabsl((long double)eff_m1[j]) / (long double)W[eff_sp[j]] / maxInv);
+    while (ldexpl(1.0L, f.eff_shift) <= m && f.eff_shift < 32) ++f.eff_shift;
+    if (f.eff_shift >= 20) ok = false;
+    f.eff.resize(eff_sp.size());
+    for (size_t j = 0; j < eff_sp.size(); ++j) {
+        f.eff[j].w = ok ? (int64_t)llroundl(ldexpl((long double)eff_m1[j] / (long double)W[eff_sp[j]] / maxInv, 62 - f.eff_shift)) : 0;
+        f.eff[j].sp = eff_sp[j];
+        f.eff[j].slot = 0;
+    }
+
+    // Ranges over the temperature window: rate constants and reaction Gibbs energies together
+    // below kMaxX (so that sums stay inside the format and a zero concentration underflows).
+    const int NT = 64;
+    std::vector<double> G(K);
+    for (int it = 0; it <= NT && ok; ++it) {
+        const double T = kFxTmin * std::pow(kFxTmax / kFxTmin, (double)it / NT), lT = std::log(T), l2e = (double)kL2E;
+        for (int k = 0; k < K; ++k) {
+            const double* a = nasa.data() + ((size_t)k * 2 + (T <= Tmid[k] ? 0 : 1)) * kNasaStride;
+            G[k] = l2e * (a[0] * (1.0 - lT) - T * (a[1] / 2 + T * (a[2] / 6 + T * (a[3] / 12 + T * a[4] / 20))) +
+                          a[5] / T - a[6] + lT) + (double)l2RP0;
+        }
+        for (int q = 0; q < R && ok; ++q) {
+            const RxnRec& r = rxn[q];
+            double g = 0.0;
+            for (int e = 0; e < r.nr; ++e) g -= r.nu[e] * G[r.sp[e]];
+            for (int e = kMaxSide; e < kMaxSide + r.np; ++e) g += r.nu[e] * G[r.sp[e]];
+            const double lk = std::fabs(l2e * (r.lnA + r.beta * lT - r.EaR / T));
+            double l0 = 0.0;
+            if (r.aux >= 0) l0 = std::fabs(l2e * (troe[r.aux].lnA0 + troe[r.aux].beta0 * lT - troe[r.aux].Ea0R / T));
+            ok = lk + std::fabs(g) < kMaxX && l0 < kMaxX;
+        }
+    }
+
+    for (int set = 0; set < kFxSets; ++set) ok = schedule(set, K, rxn, rec, spec, f.set[set]) && ok;
+    for (FxEff& e : f.eff)
+        for (int k = 0; k < (int)f.set[1].sp.size(); ++k)
+            if (f.set[1].sp[k].k == e.sp) e.slot = k;
     f.ok = ok;
     return f;
 }

@@ -10,15 +10,19 @@ namespace nk {
 
 struct FxTables {
     bool ok = false;                     // the mechanism's numbers fit the fixed-point ranges
-    int rows = 0, nchunk = 0, eff_shift = 0;
-    int image = 0, image_parts = 0, image_spec = 0, image_list = 0;
+    int eff_shift = 0;
+    struct Set {
+        FxSet s{};                       // (pointers left to the caller)
+        std::vector<unsigned char> chunks;
+        std::vector<FxSpecies> sp;
+    } set[kFxSets];
     double log2_maxinvW = 0.0;
     std::vector<uint32_t> tab;           // exp and log tables (kFxTabBytes)
-    std::vector<unsigned char> chunks;   // [nchunk][image]
     std::vector<FxExtra> extra;
     std::vector<FxTroe> troe;
-    std::vector<FxSpecies> sp;
     std::vector<FxEff> eff;
+    int th_lo = 0;                       // thermo polynomials: low range in T/2^th_lo; 0: none
+    std::vector<FxThermo> th;
 };
 
 // rxn: the mechanism's reactions in device order; nasa: [K][2][kNasaStride].

@@ -18,9 +18,6 @@
 namespace nk {
 namespace {
 
-// a rate of progress times e^d for a shift of ln A outside the fixed-point form
-static __device__ __noinline__ double fx_shift_edge(double q, double d) { return q * exp(d); }
-
 // NP parts per point, 32 points per block.  RHS: the implicit-stage sources instead (omega ->
 // W_k omega_k / rho, hrr -> hrr/(rho c_p)).  A point outside the fixed-point form (fx_T_ok,
 // fx_add_fraction, fx_point_scalars, fx_sums_bad) leaves kFxSkip in its hrr: the fallback pass
@@ -32,7 +29,8 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
                     double* __restrict__ omega, double* __restrict__ hrr) {
     extern __shared__ __align__(16) unsigned char smem_fx[];
     unsigned char* im0 = smem_fx + kFxBase + kFxScalars * 256;
-    fx_image_load(m, 0, im0);
+    const FxSet& f = m.fxs[0];
+    fx_image_load(f, 0, im0);
     const FxTab ft = stage_fx_tables(reinterpret_cast<uint32_t*>(smem_fx), m.fx_tab);
     const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem_fx + kFxTabBytes), m);   // (Troe)
     __syncthreads();
@@ -42,7 +40,7 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
     const bool live = i0 < n;
     const int64_t i = live ? i0 : n - 1;                 // idle lanes of the last block repeat point n-1
     long long* sS = reinterpret_cast<long long*>(smem_fx + kFxBase) + lane;
-    unsigned char* sP = im0 + 2 * m.fx_image + lane * 8;                         // species rows
+    unsigned char* sP = im0 + 2 * f.image + lane * 8;                         // species rows
     unsigned char* sQ = sP + (size_t)(K + 1) * kFxRow;                           // rates of progress
 
     double Ti = T[i];
@@ -53,7 +51,7 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
         unsigned long long z = 0, zc = 0;
 #pragma unroll 1
         for (int k = part; k < K; k += NP) {
-            const FxSpecies* sp = m.fx_sp + k;
+            const FxSpecies* sp = f.sp + k;
             fx_add_fraction((unsigned long long)__double_as_longlong(Y[(int64_t)__ldg(&sp->k) * ld + i]),
                             __ldg((const long long*)&sp->w), z, zc, bad);
         }
@@ -76,7 +74,7 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
         const FxFrac u = fx_frac_T(Tb);
 #pragma unroll 1
         for (int k = part; k < K; k += NP) {
-            const FxSpecies* sp = m.fx_sp + k;
+            const FxSpecies* sp = f.sp + k;
             const unsigned long long yb = (unsigned long long)__double_as_longlong(Y[(int64_t)__ldg(&sp->k) * ld + i]);
             const long long a = bad ? 0 : fx_log2_conc(yb, __ldg((const long long*)&sp->lw) + lrho, ft);
             *reinterpret_cast<long long*>(sP + k * kFxRow) = a;
@@ -95,11 +93,11 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
     double w[kFxOwn];
 #pragma unroll
     for (int j = 0; j < kFxOwn; ++j) w[j] = 0.0;
-    for (int c = 0; c < m.fx_nchunk; ++c) {
-        const unsigned char* im = im0 + (c & 1) * m.fx_image;
-        fx_image_load(m, c + 1, im0 + ((c + 1) & 1) * m.fx_image);
-        const int q1 = im[m.fx_image_parts + part + 1];
-        for (int q = im[m.fx_image_parts + part]; q < q1; ++q) {
+    for (int c = 0; c < f.nchunk; ++c) {
+        const unsigned char* im = im0 + (c & 1) * f.image;
+        fx_image_load(f, c + 1, im0 + ((c + 1) & 1) * f.image);
+        const int q1 = im[f.image_parts + part + 1];
+        for (int q = im[f.image_parts + part]; q < q1; ++q) {
             const longlong2* rec = reinterpret_cast<const longlong2*>(im + q * (int)sizeof(FxRxn));
             const longlong2 r0 = rec[0], r1 = rec[1];       // lnA, beta; Ea, (info, orig)
             const int info = (int)r1.y;
@@ -137,8 +135,8 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
             *reinterpret_cast<double*>(sQ + q * 256) = qq;
         }
         __syncthreads();
-        const uint32_t* spec = reinterpret_cast<const uint32_t*>(im + m.fx_image_spec);
-        const unsigned char* list = im + m.fx_image_list;
+        const uint32_t* spec = reinterpret_cast<const uint32_t*>(im + f.image_spec);
+        const unsigned char* list = im + f.image_list;
 #pragma unroll
         for (int j = 0; j < kFxOwn; ++j) {
             const int k = part + NP * j;
@@ -162,7 +160,7 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
 #pragma unroll 1
         for (int k = part; k < K; k += NP) {
             double o = *reinterpret_cast<const double*>(sP + k * kFxRow);
-            const FxSpecies* sp = m.fx_sp + k;
+            const FxSpecies* sp = f.sp + k;
             const int64_t* c = fx_range(sp, Ti);
             const int ks = __ldg(&sp->k);
             h = fma(fx_to_d(fx_hRT(c, P, u)), o, h);
@@ -195,7 +193,7 @@ template <int NP, bool RHS>
 cudaError_t launch_rates_fx_np(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                                const double* Y, const double* dlnA, double* omega, double* hrr, cudaStream_t s) {
     auto kern = rates_fx_kernel<NP, RHS>;
-    const size_t smem = fx_smem(m, NP, kFxRow, 256);
+    const size_t smem = fx_smem(m.fxs[0], m.K, 256);
     const cudaError_t e = ensure_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)((n + 31) / 32), 32 * NP, smem, s>>>(m, n, ld, T, p, Y, dlnA, omega, hrr);

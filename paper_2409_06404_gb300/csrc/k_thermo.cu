@@ -1,7 +1,10 @@
 // Thermodynamic properties per point: NASA-7 species c_p, h, g and the mass-based mixture
 // c_p and h, mean molar mass and ideal-gas density (Eq. 1b-1d of the paper).
-// One thread per point; species rows are read coalesced across the warp (SoA layout).
-#include "nk_internal.cuh"
+// One thread per point; species rows are read coalesced across the warp (SoA layout).  The species
+// polynomials are integer ones (nk_thermo.cuh) for 64 K <= T < 4096 K, doubles elsewhere: in
+// doubles alone the FP64 pipe bounded the kernel (25 operations per species and point, 1.04 of its
+// measured rate); four per species are left.
+#include "nk_thermo.cuh"
 
 namespace nk {
 namespace {
@@ -19,6 +22,30 @@ __global__ void __launch_bounds__(kBlk) thermo_kernel(DevMech m, int64_t n, int6
     const double Ti = T[i];
     const double lnT = log(Ti), invT = 1.0 / Ti, RT = kR * Ti;
     double s = 0.0, cp = 0.0, h = 0.0;
+    const ThT t = th_fractions(m, Ti, lnT);
+    if (t.ok) {
+        for (int k = 0; k < m.K; ++k) {
+            const FxThermo* x = m.th + k;
+            const double2 head = __ldg(reinterpret_cast<const double2*>(x));             // T_mid; sh[0], sh[1]
+            const bool lo = __double_as_longlong(Ti) <= __double_as_longlong(head.x);    // (both positive)
+            const int64_t* c = lo ? x->c[0] : x->c[1];
+            const FxFrac u = lo ? t.lo : t.hi;
+            const double yw = Y[(int64_t)k * ld + i] * __ldg(m.invW + k);
+            const double cpk = th_cp(c, u, __double2loint(head.y)), hk = th_h(c, u, __double2hiint(head.y));
+            s += yw;
+            cp = fma(yw, cpk, cp);
+            h = fma(yw, hk, h);
+            if (cp_k) cp_k[(int64_t)k * ld + i] = cpk;
+            if (h_k) h_k[(int64_t)k * ld + i] = hk;
+            if (g_k) g_k[(int64_t)k * ld + i] = th_g(c, u, t.ln, __ldg(&x->sh[2]));
+        }
+        const double wb = 1.0 / s;
+        if (cp_mix) cp_mix[i] = cp;
+        if (h_mix) h_mix[i] = h;
+        if (Wbar) Wbar[i] = wb;
+        if (rho) rho[i] = p[i] * wb * invT * kInvR;
+        return;
+    }
     for (int k = 0; k < m.K; ++k) {
         const double yw = Y[(int64_t)k * ld + i] * __ldg(m.invW + k);
         const double* c = nasa_range(m, k, Ti);

@@ -544,11 +544,13 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
                  o_mp4 = L.add(mt_ptr[1].size() * 4 + 16), o_ms2 = L.add(mt_slot[0].size() * 4 + 16),
                  o_ms4 = L.add(mt_slot[1].size() * 4 + 16), o_me2 = L.add(mt_eps[0].size() * 8 + 16),
                  o_me4 = L.add(mt_eps[1].size() * 8 + 16), o_xtab = L.add(fxt.tab.size() * 4),
-                 o_xr = L.add(fxt.chunks.size() + 16),
+                 o_xr = L.add(fxt.set[0].chunks.size() + 16), o_xr1 = L.add(fxt.set[1].chunks.size() + 16),
                  o_xx = L.add(fxt.extra.size() * sizeof(nk::FxExtra) + 16),
                  o_xt = L.add(fxt.troe.size() * sizeof(nk::FxTroe) + 16),
-                 o_xs = L.add(fxt.sp.size() * sizeof(nk::FxSpecies)),
-                 o_xe = L.add(fxt.eff.size() * sizeof(nk::FxEff) + 16);
+                 o_xs = L.add(fxt.set[0].sp.size() * sizeof(nk::FxSpecies)),
+                 o_xs1 = L.add(fxt.set[1].sp.size() * sizeof(nk::FxSpecies) + 16),
+                 o_xe = L.add(fxt.eff.size() * sizeof(nk::FxEff) + 16),
+                 o_th = L.add(fxt.th.size() * sizeof(nk::FxThermo));
     std::vector<unsigned char> host(L.bytes, 0);
     auto put = [&](size_t off, const void* src, size_t n) {
         if (n) std::memcpy(host.data() + off, src, n);
@@ -610,10 +612,13 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
     put(o_lcw, lc_w.data(), lc_w.size() * 8);
     put(o_dfe, df_effm1.data(), df_effm1.size() * 8);
     put(o_xtab, fxt.tab.data(), fxt.tab.size() * 4);
-    put(o_xr, fxt.chunks.data(), fxt.chunks.size());
+    put(o_xr, fxt.set[0].chunks.data(), fxt.set[0].chunks.size());
+    put(o_xr1, fxt.set[1].chunks.data(), fxt.set[1].chunks.size());
+    put(o_xs1, fxt.set[1].sp.data(), fxt.set[1].sp.size() * sizeof(nk::FxSpecies));
     put(o_xx, fxt.extra.data(), fxt.extra.size() * sizeof(nk::FxExtra));
     put(o_xt, fxt.troe.data(), fxt.troe.size() * sizeof(nk::FxTroe));
-    put(o_xs, fxt.sp.data(), fxt.sp.size() * sizeof(nk::FxSpecies));
+    put(o_xs, fxt.set[0].sp.data(), fxt.set[0].sp.size() * sizeof(nk::FxSpecies));
+    put(o_th, fxt.th.data(), fxt.th.size() * sizeof(nk::FxThermo));
     put(o_xe, fxt.eff.data(), fxt.eff.size() * sizeof(nk::FxEff));
 
     int dev = 0;
@@ -703,20 +708,20 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
     dm.mt_eps2 = reinterpret_cast<const double*>(b + o_me2);
     dm.mt_eps4 = reinterpret_cast<const double*>(b + o_me4);
     dm.fx_ok = fxt.ok ? 1 : 0;
-    dm.fx_rows = fxt.rows;
-    dm.fx_image = fxt.image;
-    dm.fx_image_parts = fxt.image_parts;
-    dm.fx_image_spec = fxt.image_spec;
-    dm.fx_image_list = fxt.image_list;
-    dm.fx_nchunk = fxt.nchunk;
+    dm.th_lo = fxt.th_lo;
+    dm.th = reinterpret_cast<const nk::FxThermo*>(b + o_th);
+    dm.fxs[0] = fxt.set[0].s;
+    dm.fxs[0].chunks = b + o_xr;
+    dm.fxs[0].sp = reinterpret_cast<const nk::FxSpecies*>(b + o_xs);
+    dm.fxs[1] = fxt.set[1].s;
+    dm.fxs[1].chunks = b + o_xr1;
+    dm.fxs[1].sp = reinterpret_cast<const nk::FxSpecies*>(b + o_xs1);
     dm.fx_eff_shift = fxt.eff_shift;
     dm.fx_lmaxw = (int64_t)llroundl((long double)fxt.log2_maxinvW * 281474976710656.0L);
     dm.fx_lR = (int64_t)llroundl(log2l((long double)nk::kR) * 281474976710656.0L);
     dm.fx_tab = reinterpret_cast<const uint32_t*>(b + o_xtab);
-    dm.fx_chunks = b + o_xr;
     dm.fx_extra = reinterpret_cast<const nk::FxExtra*>(b + o_xx);
     dm.fx_troe = reinterpret_cast<const nk::FxTroe*>(b + o_xt);
-    dm.fx_sp = reinterpret_cast<const nk::FxSpecies*>(b + o_xs);
     dm.fx_eff = reinterpret_cast<const nk::FxEff*>(b + o_xe);
     dm.mslots2 = mslots[0];
     dm.mslots4 = mslots[1];

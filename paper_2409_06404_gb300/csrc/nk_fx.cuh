@@ -160,6 +160,16 @@ __device__ __forceinline__ double fx_to_d(long long x) {
     const unsigned long long b = m + ((unsigned long long)(1023 + 63 - kFxS - z - 1) << 52);
     return __longlong_as_double((long long)(b | ((unsigned long long)x & 0x8000000000000000ull)));
 }
+// x 2^-s as a double (to nearest, ties up in magnitude), by integer operations
+__device__ __forceinline__ double fx_round_d(long long x, int s) {
+    const unsigned long long a = (unsigned long long)(x < 0 ? -x : x);
+    if (a == 0) return 0.0;
+    const int z = __clzll((long long)a);
+    const unsigned long long n = a << z;
+    const unsigned long long m = (n >> 11) + ((n >> 10) & 1ull);                      // 53 bits (a carry raises the exponent)
+    const unsigned long long b = m + ((unsigned long long)(1023 + 63 - s - z - 1) << 52);
+    return __longlong_as_double((long long)(b | ((unsigned long long)x & 0x8000000000000000ull)));
+}
 // x 2^-48 as a float pair (pieces of 22 bits, exact but for the last rounding)
 __device__ __forceinline__ dfl fx_to_pair(long long x) {
     const float a = __fmul_rn(__fsub_rn(__int_as_float(0x4B400000 + (int)(x >> 44)), 12582912.0f), 0x1p-4f);

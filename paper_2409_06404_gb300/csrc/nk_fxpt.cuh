@@ -83,19 +83,19 @@ __device__ __forceinline__ const int64_t* fx_range(const FxSpecies* s, double T)
 constexpr int kFxScalars = 5;      // log2 T, 128/T (63 bits), log2(p/(R T)), log2 rho', sum Y/W
 enum { kFxLT = 0, kFxV = 1, kFxLpRT = 2, kFxLrho = 3, kFxSum = 4 };
 constexpr size_t kFxBase = kFxTabBytes + kDfTabBytes;
-// species_bytes: bytes per species row (kFxRow, more for the derivatives); the row after the last
-// species is zero.  Two chunk images are double buffered.
-inline size_t fx_smem(const DevMech& m, int NP, int species_bytes, int row_bytes) {
-    const size_t q = (size_t)m.fx_rows * row_bytes, part = (size_t)NP * 2 * 256;   // the parts' sums come first
-    return kFxBase + kFxScalars * 256 + 2 * (size_t)m.fx_image + (size_t)species_bytes * (m.K + 1) + (q > part ? q : part);
+// The row after the last species is zero; two chunk images are double buffered; row_bytes per
+// reaction of a chunk.
+inline size_t fx_smem(const FxSet& f, int K, int row_bytes) {
+    const size_t q = (size_t)f.rows * row_bytes, part = (size_t)f.np * 3 * 256;   // the parts' sums come first
+    return kFxBase + kFxScalars * 256 + 2 * (size_t)f.image + (size_t)f.row * (K + 1) + (q > part ? q : part);
 }
 // Starts the copy of chunk c's image into shared memory (cp.async; waited for by fx_image_wait and
 // a barrier).
-__device__ __forceinline__ void fx_image_load(const DevMech& m, int c, unsigned char* dst) {
-    if (c < m.fx_nchunk) {
-        const unsigned char* src = m.fx_chunks + (size_t)c * m.fx_image;
+__device__ __forceinline__ void fx_image_load(const FxSet& f, int c, unsigned char* dst) {
+    if (c < f.nchunk) {
+        const unsigned char* src = f.chunks + (size_t)c * f.image;
         const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-        for (int o = threadIdx.x * 16; o < m.fx_image; o += blockDim.x * 16)
+        for (int o = threadIdx.x * 16; o < f.image; o += blockDim.x * 16)
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d + o), "l"(src + o) : "memory");
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -258,16 +258,20 @@ __device__ __forceinline__ FxRate fx_sides(const unsigned char* sp, int info, ui
     return x;
 }
 
-// Sum over one species' rows of a chunk (w: its word in the image, list: the image's row list, q:
+// a rate of progress times e^d for a shift of ln A outside the fixed-point form
+static __device__ __noinline__ double fx_shift_edge(double q, double d) { return q * exp(d); }
+
+// Sum over one species' rows of a chunk, the rows MUL 256 bytes apart (w: its word in the image, list: the image's row list, q:
 // the rows, this lane's column), added to s in list order.
+template <int MUL = 1>
 __device__ __forceinline__ double fx_gather(uint32_t w, const unsigned char* list, const unsigned char* q, double s) {
     const unsigned char* l = list + (w >> 15 & ~1u);
     const unsigned char* e = l + (w >> 7 & 510u);
 #pragma unroll 1
-    for (; l != e; l += 2) s += *reinterpret_cast<const double*>(q + *reinterpret_cast<const uint16_t*>(l));
+    for (; l != e; l += 2) s += *reinterpret_cast<const double*>(q + MUL * *reinterpret_cast<const uint16_t*>(l));
     e += (w & 255u) * 2;
 #pragma unroll 1
-    for (; l != e; l += 2) s -= *reinterpret_cast<const double*>(q + *reinterpret_cast<const uint16_t*>(l));
+    for (; l != e; l += 2) s -= *reinterpret_cast<const double*>(q + MUL * *reinterpret_cast<const uint16_t*>(l));
     return s;
 }
 

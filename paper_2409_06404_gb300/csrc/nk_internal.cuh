@@ -96,11 +96,12 @@ struct __align__(16) JacTerm {
 
 // Fixed-point tables (nk_fx.cuh, built by fx_tables.cu): logarithms to base 2 in units of 2^-48.
 // One reaction: ln k_f = lnA + beta lt + Ea v with fx_mul and the point's fractions of log2 T and
-// 1/T; off: byte offsets of its molecules' rows (kFxRow per species slot; a coefficient nu repeats its
+// 1/T; off: byte offsets of its molecules' rows (FxSet::row per species slot; a coefficient nu repeats its
 // species), reactants at [0, nr), products at [4, 4 + np); the first two of each side always name
 // a row (the row after the last species holds zeros).  info = nr | np << 4 | kind << 8 |
 // index of the FxExtra record (third-body and Troe) << 16.
-constexpr int kFxRow = 512;       // a species' row: log2 C_k and mu_k of 32 points
+constexpr int kFxRow = 512;       // a species' row in the rates kernel: log2 C_k and mu_k of 32 points
+constexpr int kFxDRow = 1280;     // and in the derivative kernels
 struct __align__(16) FxRxn {
     int64_t lnA, beta, Ea;
     int32_t info, orig;
@@ -110,12 +111,24 @@ static_assert(sizeof(FxRxn) == 64, "fixed-point reaction record");
 struct __align__(16) FxExtra {
     int32_t eff0, eff1, aux, pad;  // third-body efficiencies [eff0, eff1), Troe record or -1
 };
-// Chunks: up to kFxChunk reactions whose rates of progress are staged together.  A chunk's image
+// Chunks: up to FxSet::chunk reactions whose rates of progress are staged together.  A chunk's image
 // (fx_image bytes, a multiple of 16) holds its reaction records in schedule order (part by part,
 // balanced by cost), then at image_parts the first record of each part (NP + 1 bytes), at
 // image_spec one word per species slot (start in the list << 16 | rows to add << 8 | rows to
 // subtract) and at image_list the rows as 16-bit byte offsets (256 per row).
-constexpr int kFxChunk = 48;
+// NASA-7 polynomials of one species as 64-bit integers (thermo and diffusion kernels), per range in
+// u = T/2^(b + 1) (b: DevMech::th_lo for the low range, 12 for the high one; fx_mul halves): c_p in
+// J/(mol K) (c[0..4]), h in J/mol (c[5..10]: constant, u..u^5) and g in J/mol (c[11..17]: constant,
+// then inside a factor u: constant, ln(T)/16, u..u^4), in units of 2^-sh[0], 2^-sh[1] and
+// 2^-sh[2], each as fine as its largest coefficient allows (the last bit is below a double's).
+struct __align__(16) FxThermo {
+    double Tmid;
+    int32_t sh[3], pad;
+    int64_t pad2;
+    int64_t c[2][18];
+};
+static_assert(sizeof(FxThermo) == 320, "thermo record");
+
 // One Troe reaction: its low-pressure limit as FxRxn's, and F_cent's terms: log2(1 - a),
 // -log2(e)/T3 times T, log2 a, -log2(e)/T1 times T and -log2(e) T2 times 1/T (flags: 1 the terms
 // fit, 2 the last one is there).
@@ -137,10 +150,19 @@ struct __align__(16) FxSpecies {
 };
 struct __align__(16) FxEff {
     int64_t w;          // (eps - 1)/W relative to the largest 1/W, units 2^(eff_shift - 62)
-    int32_t sp, pad;
+    int32_t sp, slot;   // species, and its slot in the derivative kernels
 };
 
 constexpr int kTroeDf = 4;       // float4 records per Troe reaction in DevMech::troe_df
+
+// The schedule of one kernel family: parts per point, the largest chunk's reactions, chunks, bytes
+// of a chunk image and of its pieces, bytes of a species row, and the species in slot order.
+struct FxSet {
+    int32_t np, rows, nchunk, image, image_parts, image_spec, image_list, row;
+    const unsigned char* chunks;      // [nchunk][image]
+    const FxSpecies* sp;              // [K]
+};
+constexpr int kFxSets = 2;            // 0: rates; 1: derivatives
 
 // Device view of a loaded mechanism (passed by value to every kernel).
 struct DevMech {
@@ -231,15 +253,16 @@ struct DevMech {
     const double* lc_w;           // [R][2 kMaxSide]
     const float2* df_eff_m1;      // efficiencies - 1 as pairs (eff_m1 order)
     // fixed-point tables of the FP64 reaction kernels (fx_ok: the mechanism fits them)
-    int32_t fx_ok, fx_rows, fx_nchunk, fx_eff_shift;      // fx_rows: the largest chunk's reactions
-    int32_t fx_image, fx_image_parts, fx_image_spec, fx_image_list;
+    int32_t fx_ok, fx_eff_shift;
+    FxSet fxs[kFxSets];
     int64_t fx_lmaxw, fx_lR;      // log2(largest 1/W), log2(R)
     const uint32_t* fx_tab;
-    const unsigned char* fx_chunks;   // [fx_nchunk][fx_image]
     const FxExtra* fx_extra;
     const FxTroe* fx_troe;
-    const FxSpecies* fx_sp;           // [K] in slot order
     const FxEff* fx_eff;
+    // fixed-point thermo polynomials (th_lo: low-range fraction T/2^th_lo; 0: they do not fit)
+    int32_t th_lo, th_pad;
+    const FxThermo* th;
 };
 
 // Centre of the re-expanded transport fits (ln T about 1100 K).
@@ -257,8 +280,13 @@ struct JitModule {
 
 namespace nk {
 constexpr int kFxOwn = 8;          // species per part of the fixed-point kernels, at most
-// Parts (warps) per point for K species.
-inline int fx_parts(int K) { return K <= 4 * kFxOwn ? 4 : K <= 8 * kFxOwn ? 8 : K <= 16 * kFxOwn ? 16 : 32; }
+// Parts (warps) per point for K species: the rates kernel takes 64 registers and as many blocks as
+// make 32 warps per SM; the derivative kernels 80 registers, 24 warps (6, 2 or 1 blocks: their
+// species rows fill shared memory; 0: they do not fit).
+inline int fx_parts(int K, int set = 0) {
+    if (set == 0) return K <= 4 * kFxOwn ? 4 : K <= 8 * kFxOwn ? 8 : K <= 16 * kFxOwn ? 16 : 32;
+    return K <= 32 ? 4 : K <= 64 ? 12 : K <= 140 ? 24 : 0;
+}
 }  // namespace nk
 
 // The opaque handle of the public ABI.
