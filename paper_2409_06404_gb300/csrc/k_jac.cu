@@ -39,11 +39,27 @@
 namespace nk {
 namespace {
 
-// 2^-e with the largest |entry| m = f 2^e, f in [1/2, 1); e = 0 for a zero or non-finite m
-__device__ __forceinline__ int row_exponent(double m) {
-    int e = 0;
-    if (m > 0.0 && m <= 1.7976931348623157e308) frexp(m, &e);
+// e with the largest |entry| m = f 2^e, f in [1/2, 1), from m's bits; 0 for a zero or infinite m
+__device__ __forceinline__ int row_exponent(unsigned long long m) {
+    int e = (int)(m >> 52) - 1022;
+    if (m == 0 || m >= 0x7ff0000000000000ull) return 0;
+    if (m < 0x0010000000000000ull) frexp(__longlong_as_double((long long)m), &e);
     return e;
+}
+
+// the larger of a magnitude (bits; non-negative doubles order as integers) and |v|, NaN ignored:
+// comparisons of doubles run on the FP64 pipe, which bounds the kernel
+__device__ __forceinline__ unsigned long long max_mag(unsigned long long m, double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+    return b > m && b <= 0x7ff0000000000000ull ? b : m;
+}
+
+// v 2^-e on the bits where the result is normal (or v is zero)
+__device__ __forceinline__ double scale_down(double v, int e, double sc) {
+    const int x = (int)((unsigned)__double2hiint(v) >> 20 & 0x7ffu);
+    if (x != 0 && x != 0x7ff && x - e > 0 && x - e < 0x7ff)
+        return __hiloint2double(__double2hiint(v) - (e << 20), __double2loint(v));
+    return (__double_as_longlong(v) << 1) == 0 ? v : v * sc;
 }
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -52,10 +68,9 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__device__ __forceinline__ double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+__device__ __forceinline__ unsigned long long warp_max(unsigned long long v) {
+    const unsigned h = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32));
+    return (unsigned long long)h << 32 | __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == h ? (unsigned)v : 0u);
 }
 
 // doubles of shared memory per point: N (N + 1) block entries, 6K + 8 of vectors, 2N ints
@@ -159,16 +174,16 @@ __global__ void block_kernel(const DevMech m, const int64_t n, const int64_t ld,
             if constexpr (PREC) {
                 const double rw = out.dt * out.w[(int64_t)(k + 1) * out.ldw + i];   // dt w_(k+1)
                 const double vT = -rw * jT * iw0, rf = rw * Wk;
-                double mx = fabs(vT);
+                unsigned long long mx = max_mag(0, vT);
                 ar[0] = vT;
                 for (int j = 0; j < K; ++j) {
                     const double v = (k == j ? 1.0 : 0.0) - rf * (ar[j + 1] - ck) * colf[j];
                     ar[j + 1] = v;
-                    mx = fmax(mx, fabs(v));
+                    mx = max_mag(mx, v);
                 }
                 const int e = row_exponent(mx);
                 const double sc = ldexp(1.0, -e);
-                for (int j = 0; j < N; ++j) ar[j] *= sc;
+                for (int j = 0; j < N; ++j) ar[j] = scale_down(ar[j], e, sc);
                 ex[k + 1] = e;
             } else {
                 ar[0] = jT;
@@ -178,7 +193,7 @@ __global__ void block_kernel(const DevMech m, const int64_t n, const int64_t ld,
         // temperature row
         const double RT = kR * Ti, icp = irho / cpm, icpm = 1.0 / cpm, is = 1.0 / s;
         const double rT = PREC ? out.dt * out.w[i] : 1.0;
-        double mx = 0.0;
+        unsigned long long mx = 0;
         for (int j = lane; j < K; j += 32) {
             const double iw = __ldg(m.invW + j);
             const double aj = -iw * is;
@@ -188,7 +203,7 @@ __global__ void block_kernel(const DevMech m, const int64_t n, const int64_t ld,
             if constexpr (PREC) {
                 const double qv = -rT * v * __ldg(m.W + j) * colf[j];
                 a[j + 1] = qv;
-                mx = fmax(mx, fabs(qv));
+                mx = max_mag(mx, qv);
             } else {
                 a[j + 1] = v;
             }
@@ -198,10 +213,10 @@ __global__ void block_kernel(const DevMech m, const int64_t n, const int64_t ld,
         const double jTT = icp * fma(-hrr, fma(dcpm, icpm, -invT), dhT);
         if constexpr (PREC) {
             const double vTT = 1.0 - out.dt * jTT;
-            mx = fmax(warp_max(mx), fabs(vTT));
+            mx = max_mag(warp_max(mx), vTT);
             const int e0 = row_exponent(mx);
             const double sc0 = ldexp(1.0, -e0);
-            for (int j = lane; j < K; j += 32) a[j + 1] *= sc0;
+            for (int j = lane; j < K; j += 32) a[j + 1] = scale_down(a[j + 1], e0, sc0);
             if (lane == 0) {
                 a[0] = vTT * sc0;
                 ex[0] = e0;
