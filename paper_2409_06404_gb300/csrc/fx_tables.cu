@@ -41,12 +41,13 @@ const std::vector<uint32_t>& math_tables() {
 
 // One kernel family's schedule: species slots and chunk images.
 bool schedule(int set, int K, const std::vector<RxnRec>& rxn, const std::vector<FxRxn>& rec,
-              const std::vector<FxSpecies>& species, FxTables::Set& out) {
+              const std::vector<FxSpecies>& species, const std::vector<int32_t>& eff_sp,
+              const std::vector<double>& eff_w, FxTables::Set& out) {
     const int R = (int)rxn.size(), NP = fx_parts(K, set);
     FxSet& f = out.s;
     bool ok = true;
     f.np = NP;
-    f.row = set == 0 ? kFxRow : kFxDRow;
+    f.row = set == 0 ? kFxRow : set == 1 ? kFxDRow : 256;
     if (NP == 0) return true;              // (the family does not take this mechanism)
 
     // species slots: by decreasing number of molecules over all reactions, dealt to the parts with
@@ -73,7 +74,7 @@ bool schedule(int set, int K, const std::vector<RxnRec>& rxn, const std::vector<
 
     // Chunks of about equal size with the costlier kinds spread evenly over them; within a chunk
     // the reactions go to the parts by decreasing cost, each to the part with the least so far.
-    const int chunk = set == 0 ? 48 : 48;
+    const int chunk = set != 1 || NP > 12 ? 48 : 36;   // (derivatives: their rows share the memory)
     f.nchunk = (R + chunk - 1) / chunk;
     std::vector<std::vector<int>> members(f.nchunk);
     for (int kind = 2, next = 0; kind >= 0; --kind)
@@ -83,7 +84,8 @@ bool schedule(int set, int K, const std::vector<RxnRec>& rxn, const std::vector<
     std::vector<std::vector<int>> order(f.nchunk);
     std::vector<std::vector<unsigned char>> first(f.nchunk);
     std::vector<std::vector<std::vector<uint16_t>>> add(f.nchunk), sub(f.nchunk);
-    size_t most = 0;
+    std::vector<std::vector<std::vector<FxEffTerm>>> effs(f.nchunk);
+    size_t most = 0, most_eff = 0;
     for (int c = 0; c < f.nchunk; ++c) {
         std::vector<std::vector<int>> part(NP);
         std::vector<int> load(NP, 0);
@@ -100,9 +102,15 @@ bool schedule(int set, int K, const std::vector<RxnRec>& rxn, const std::vector<
         f.rows = std::max(f.rows, (int)order[c].size());
         add[c].resize(K);
         sub[c].resize(K);
-        size_t entries = 0;
+        size_t entries = 0, neff = 0;
+        effs[c].resize(K);
+        int nx = 0;
         for (size_t i = 0; i < order[c].size(); ++i) {
             const RxnRec& r = rxn[order[c][i]];
+            if (r.type != NK_RXN_ELEMENTARY) {
+                for (int j = r.eff0; j < r.eff1; ++j, ++neff) effs[c][slot[eff_sp[j]]].push_back(FxEffTerm{eff_w[j], nx, 0});
+                ++nx;
+            }
             for (int side = 0; side < 2; ++side)
                 for (int e = 0; e < (side ? r.np : r.nr); ++e)
                     for (int j = 0; j < r.nu[side * kMaxSide + e]; ++j, ++entries)
@@ -110,19 +118,35 @@ bool schedule(int set, int K, const std::vector<RxnRec>& rxn, const std::vector<
         }
         for (int k = 0; k < K; ++k) ok = ok && add[c][k].size() < 256 && sub[c][k].size() < 256;
         most = std::max(most, entries);
+        most_eff = std::max(most_eff, neff);
+        f.xrows = std::max(f.xrows, nx);
     }
     auto up = [](int v) { return (v + 15) / 16 * 16; };
     f.image_parts = f.rows * (int)sizeof(FxRxn);
     f.image_spec = f.image_parts + up(NP + 1);
     f.image_list = f.image_spec + up(4 * K);
-    f.image = f.image_list + up(2 * (int)most);
+    f.image_eff = f.image_list + up(2 * (int)most);
+    f.image_effl = f.image_eff + (set != 1 ? 0 : up(4 * K));
+    f.image = f.image_effl + (set != 1 ? 0 : (int)(most_eff * sizeof(FxEffTerm)));
+    ok = ok && f.xrows < 64;
     out.chunks.assign((size_t)f.nchunk * f.image, 0);
     for (int c = 0; c < f.nchunk; ++c) {
         unsigned char* im = out.chunks.data() + (size_t)c * f.image;
+        int nx = 0;
         for (size_t i = 0; i < order[c].size(); ++i) {
             FxRxn x = rec[order[c][i]];
             for (uint32_t& o : x.off) o = (o == (uint32_t)K ? (uint32_t)K : (uint32_t)slot[o]) * (uint32_t)f.row;
+            if (rxn[order[c][i]].type != NK_RXN_ELEMENTARY) x.info |= (nx++ & 63) << 10;
             std::memcpy(im + i * sizeof(FxRxn), &x, sizeof x);
+        }
+        if (set == 1) {
+            uint32_t at = 0;
+            for (int k = 0; k < K; ++k) {
+                ok = ok && effs[c][k].size() < 256;
+                const uint32_t w = at << 8 | (uint32_t)(effs[c][k].size() & 255);
+                std::memcpy(im + f.image_eff + 4 * k, &w, 4);
+                for (const FxEffTerm& t : effs[c][k]) std::memcpy(im + f.image_effl + (at++) * sizeof(FxEffTerm), &t, sizeof t);
+            }
         }
         std::memcpy(im + f.image_parts, first[c].data(), NP + 1);
         uint32_t at = 0;
@@ -136,11 +160,72 @@ bool schedule(int set, int K, const std::vector<RxnRec>& rxn, const std::vector<
     return ok;
 }
 
+// The single-precision products' chunks of consecutive reactions of `order`.
+bool schedule32(int K, const std::vector<RxnRec>& rxn, const std::vector<int>& order, const std::vector<int32_t>& boff,
+                const std::vector<int32_t>& slot, FxTables::Set& out) {
+    const int R = (int)order.size(), NP = fx_parts(K, 2), chunk = 48;
+    FxSet& f = out.s;
+    bool ok = true;
+    f.np = NP;
+    f.row = 128;
+    f.nchunk = (R + chunk - 1) / chunk;
+    const int per = (R + f.nchunk - 1) / f.nchunk;
+    f.rows = per;
+    std::vector<std::vector<std::vector<FxTerm32>>> terms(f.nchunk);
+    size_t most = 0;
+    auto up = [](int v) { return (v + 15) / 16 * 16; };
+    for (int c = 0; c < f.nchunk; ++c) {
+        terms[c].resize(K);
+        size_t n = 0;
+        for (int i = c * per; i < std::min(R, (c + 1) * per); ++i) {
+            const RxnRec& r = rxn[order[i]];
+            for (int side = 0; side < 2; ++side)
+                for (int e = 0; e < (side ? r.np : r.nr); ++e, ++n)
+                    terms[c][slot[r.sp[side * kMaxSide + e]]].push_back(
+                        FxTerm32{(uint32_t)(i - c * per) * 256u, (float)r.nud[side * kMaxSide + e]});
+        }
+        most = std::max(most, n);
+    }
+    f.image_parts = per * (int)sizeof(FxRxn32);
+    f.image_spec = f.image_parts + up(NP + 1);
+    f.image_list = f.image_spec + up(4 * K);
+    f.image = f.image_list + up((int)(most * sizeof(FxTerm32)));
+    out.chunks.assign((size_t)f.nchunk * f.image, 0);
+    for (int c = 0; c < f.nchunk; ++c) {
+        unsigned char* im = out.chunks.data() + (size_t)c * f.image;
+        const int n = std::min(R, (c + 1) * per) - c * per;
+        for (int i = 0; i < n; ++i) {
+            const int q = order[c * per + i];
+            const RxnRec& r = rxn[q];
+            FxRxn32 x;
+            std::memset(&x, 0, sizeof x);
+            for (int e = 0; e < r.nr; ++e) x.off[e] = (uint16_t)(slot[r.sp[e]] * 128);
+            for (int e = 0; e < r.np; ++e) x.off[4 + e] = (uint16_t)(slot[r.sp[kMaxSide + e]] * 128);
+            x.info = r.nr | r.np << 4 | r.type << 8;
+            x.r = q;
+            x.boff = boff[q];
+            x.eff0 = r.eff0;
+            x.eff1 = r.eff1;
+            std::memcpy(im + i * sizeof x, &x, sizeof x);
+        }
+        for (int p = 0; p <= NP; ++p) im[f.image_parts + p] = (unsigned char)(n * p / NP);
+        uint32_t at = 0;
+        for (int k = 0; k < K; ++k) {
+            ok = ok && terms[c][k].size() < 256;
+            const uint32_t w = at << 8 | (uint32_t)(terms[c][k].size() & 255);
+            std::memcpy(im + f.image_spec + 4 * k, &w, 4);
+            for (const FxTerm32& t : terms[c][k]) std::memcpy(im + f.image_list + (at++) * sizeof t, &t, sizeof t);
+        }
+    }
+    return ok;
+}
+
 }  // namespace
 
 FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vector<TroeRec>& troe,
                          const std::vector<int32_t>& eff_sp, const std::vector<double>& eff_m1,
-                         const std::vector<double>& nasa, const double* W, const double* Tmid) {
+                         const std::vector<double>& nasa, const double* W, const double* Tmid,
+                         const std::vector<int> (&order32)[3], const std::vector<int32_t>& lin_boff) {
     FxTables f;
     const int R = (int)rxn.size();
     bool ok = true;
@@ -244,7 +329,8 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
         x.lnA = put(kL2E * r.lnA) + 2;    // (fx_mul cuts about 1.25 units)
         x.beta = put(32.0L * r.beta);
         x.Ea = put(-kL2E * r.EaR / 64.0L);
-        x.orig = r.orig;
+        x.orig = r.orig | q << 16;
+        f.nu1.push_back(r.nu[0] | r.nu[kMaxSide] << 4);
         int cnt[2] = {0, 0};
         for (int e = 0; e < 8; ++e) x.off[e] = (uint32_t)K;          // (species; offsets per set below)
         for (int side = 0; side < 2; ++side) {
@@ -284,11 +370,16 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
         m = std::max(m, fabsl((long double)eff_m1[j]) / (long double)W[eff_sp[j]] / maxInv);
     while (ldexpl(1.0L, f.eff_shift) <= m && f.eff_shift < 32) ++f.eff_shift;
     if (f.eff_shift >= 20) ok = false;
+    std::vector<double> eff_w(eff_sp.size());
+    for (size_t j = 0; j < eff_sp.size(); ++j)
+        eff_w[j] = (double)((long double)eff_m1[j] / (long double)W[eff_sp[j]] / maxInv);
     f.eff.resize(eff_sp.size());
     for (size_t j = 0; j < eff_sp.size(); ++j) {
         f.eff[j].w = ok ? (int64_t)llroundl(ldexpl((long double)eff_m1[j] / (long double)W[eff_sp[j]] / maxInv, 62 - f.eff_shift)) : 0;
         f.eff[j].sp = eff_sp[j];
-        f.eff[j].slot = 0;
+        f.eff[j].pad = 0;
+        f.eff[j].wd = eff_w[j];
+        f.eff[j].pad2 = 0;
     }
 
     // Ranges over the temperature window: rate constants and reaction Gibbs energies together
@@ -314,10 +405,10 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
         }
     }
 
-    for (int set = 0; set < kFxSets; ++set) ok = schedule(set, K, rxn, rec, spec, f.set[set]) && ok;
-    for (FxEff& e : f.eff)
-        for (int k = 0; k < (int)f.set[1].sp.size(); ++k)
-            if (f.set[1].sp[k].k == e.sp) e.slot = k;
+    for (int set = 0; set < kFxSets; ++set) ok = schedule(set, K, rxn, rec, spec, eff_sp, eff_w, f.set[set]) && ok;
+    f.slot32.assign(K, 0);
+    for (int q = 0; q < K; ++q) f.slot32[f.set[2].sp[q].k] = q;
+    for (int v = 0; v < 3; ++v) ok = schedule32(K, rxn, order32[v], lin_boff, f.slot32, f.set32[v]) && ok;
     f.ok = ok;
     return f;
 }

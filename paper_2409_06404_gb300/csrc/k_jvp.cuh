@@ -25,6 +25,7 @@
 #include <utility>
 #include <vector>
 
+#include "k_jvp_fx.cuh"
 #include "nk_rxn.cuh"
 
 namespace nk {
@@ -306,8 +307,9 @@ __device__ __forceinline__ void jvp_rounds(const DevMech& m, int part, bool dire
 __host__ __device__ constexpr int jvp_rows(bool omega) { return omega ? 4 : 3; }
 
 // RHS: the JVP of the implicit-stage sources (omega -> W_k omega_k / rho, hrr -> hrr/(rho c_p)
-// and their tangents in d_omega, d_hrr).
-template <int BLK, int NP, bool OMEGA, bool RHS>
+// and their tangents in d_omega, d_hrr).  MARKED: only the points whose d_hrr holds kFxSkip (left by
+// the fixed-point kernel, k_jvp_fx.cuh, which takes the others).
+template <int BLK, int NP, bool OMEGA, bool RHS, bool MARKED = false>
 __global__ void __launch_bounds__(BLK * NP, 512 / (BLK * NP)) jvp_kernel(const DevMech m, const int64_t n, const int64_t ld,
                                                        const double* __restrict__ T, const double* __restrict__ p,
                                                        const double* __restrict__ Y, const double* __restrict__ dlnA,
@@ -321,8 +323,13 @@ __global__ void __launch_bounds__(BLK * NP, 512 / (BLK * NP)) jvp_kernel(const D
     const int slot = threadIdx.x % BLK, part = threadIdx.x / BLK;
     const int64_t i0 = (int64_t)blockIdx.x * BLK + slot;
     if (NP == 1 && i0 >= n) return;              // (NP = 1 has no barrier below)
-    const bool live = i0 < n;
+    bool live = i0 < n;
     const int64_t i = live ? i0 : n - 1;         // idle slots of the last block recompute point n-1
+    if constexpr (MARKED) {
+        const bool marked = __double_as_longlong(d_hrr[i]) == (long long)kFxSkip;
+        if (!(NP > 1 ? __syncthreads_or(marked) != 0 : __any_sync(__activemask(), marked))) return;
+        live &= marked;
+    }
     double* base = smem + kMathTabDoubles + slot;
     double* sC = base;                                   // C_k
     double* sdC = base + (size_t)K * BLK;                // dC_k
@@ -496,6 +503,20 @@ size_t jvp_smem(int K, const Shape& sh, bool omega) {
     return (size_t)kMathTabDoubles * sizeof(double) + (size_t)jvp_rows(omega) * K * sh.blk * sizeof(double);
 }
 
+// The marked points of the fixed-point kernel.
+template <bool OMEGA, bool RHS>
+cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
+                          const double* dlnA, const double* vT, const double* vY, double* omega, double* hrr,
+                          double* d_omega, double* d_hrr, cudaStream_t st) {
+    const Shape sh{32, m.K >= 12 ? 4 : 1};
+    const size_t smem = jvp_smem(m.K, sh, OMEGA);
+    auto kern = sh.np == 4 ? jvp_kernel<32, 4, OMEGA, RHS, true> : jvp_kernel<32, 1, OMEGA, RHS, true>;
+    const cudaError_t e = ensure_smem((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((n + 31) / 32), 32 * sh.np, smem, st>>>(m, n, ld, T, p, Y, dlnA, vT, vY, omega, hrr, d_omega, d_hrr);
+    return cudaGetLastError();
+}
+
 struct Plan {
     int dev, K;
     bool omega, rhs;
@@ -566,6 +587,10 @@ template <bool OMEGA, bool RHS>
 cudaError_t launch_o(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
                      const double* dlnA, const double* vT, const double* vY, double* omega, double* hrr,
                      double* d_omega, double* d_hrr, cudaStream_t s) {
+    if (jvp_fx_fits(m, OMEGA)) {
+        const cudaError_t e = launch_jvp_fx<OMEGA, RHS>(m, n, ld, T, p, Y, dlnA, vT, vY, omega, hrr, d_omega, d_hrr, s);
+        return e != cudaSuccess ? e : launch_marked<OMEGA, RHS>(m, n, ld, T, p, Y, dlnA, vT, vY, omega, hrr, d_omega, d_hrr, s);
+    }
     const int idx = plan_shape<OMEGA, RHS>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
     return launch_idx<OMEGA, RHS>(idx, std::make_integer_sequence<int, kNumShapes>{}, m, n, ld, T, p, Y, dlnA, vT,

@@ -106,13 +106,13 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
             long long shift = 0;
             bool big = false;                               // a shift of ln A outside +-2048 (or NaN)
             if (dlnA) {
-                const double d = __ldg(dlnA + (int)(r1.y >> 32));
+                const double d = __ldg(dlnA + (int)(r1.y >> 32 & 0xffff));
                 big = ((unsigned)__double2hiint(d) & 0x7fffffffu) >= 0x40a00000u;
                 if (!big) shift = fx_log2e_times(d);
                 lnk += shift;
             }
             long long z = 1;                                // [M]/rho' of third-body and Troe reactions
-            const int kind = info >> 8 & 255;
+            const int kind = info >> 8 & 3;
             if (kind != 0) {
                 const int4 x = __ldg(reinterpret_cast<const int4*>(m.fx_extra + (info >> 16)));
                 long long lM;
@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
             L.f += lnk;
             double qq = fx_exp2<true>(L.f, ft) - fx_exp2<true>(L.f + L.r, ft);
             if (z <= 0 && (z == 0 || kind == 2)) qq = z == 0 ? 0.0 : __longlong_as_double(0x7ff8000000000000ll);
-            if (big) qq = fx_shift_edge(qq, __ldg(dlnA + (int)(r1.y >> 32)));
+            if (big) qq = fx_shift_edge(qq, __ldg(dlnA + (int)(r1.y >> 32 & 0xffff)));
             *reinterpret_cast<double*>(sQ + q * 256) = qq;
         }
         __syncthreads();

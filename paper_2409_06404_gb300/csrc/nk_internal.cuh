@@ -98,8 +98,9 @@ struct __align__(16) JacTerm {
 // One reaction: ln k_f = lnA + beta lt + Ea v with fx_mul and the point's fractions of log2 T and
 // 1/T; off: byte offsets of its molecules' rows (FxSet::row per species slot; a coefficient nu repeats its
 // species), reactants at [0, nr), products at [4, 4 + np); the first two of each side always name
-// a row (the row after the last species holds zeros).  info = nr | np << 4 | kind << 8 |
-// index of the FxExtra record (third-body and Troe) << 16.
+// a row (the row after the last species holds zeros).  info = nr | np << 4 | kind << 8 | (third-body
+// and Troe) its number among the chunk's << 10 | index of its FxExtra record << 16; orig = caller's
+// index | device order << 16.
 constexpr int kFxRow = 512;       // a species' row in the rates kernel: log2 C_k and mu_k of 32 points
 constexpr int kFxDRow = 1280;     // and in the derivative kernels
 struct __align__(16) FxRxn {
@@ -115,7 +116,13 @@ struct __align__(16) FxExtra {
 // (fx_image bytes, a multiple of 16) holds its reaction records in schedule order (part by part,
 // balanced by cost), then at image_parts the first record of each part (NP + 1 bytes), at
 // image_spec one word per species slot (start in the list << 16 | rows to add << 8 | rows to
-// subtract) and at image_list the rows as 16-bit byte offsets (256 per row).
+// subtract) and at image_list the rows as 16-bit byte offsets (256 per row).  For the derivative
+// kernels image_eff holds one word per species slot (start << 8 | count) of its third-body
+// efficiencies in the chunk, listed at image_effl (FxEffTerm).
+struct __align__(16) FxEffTerm {
+    double w;           // (eps - 1)/W relative to the largest 1/W
+    int32_t x, pad;     // number of the reaction among the chunk's third-body and Troe reactions
+};
 // NASA-7 polynomials of one species as 64-bit integers (thermo and diffusion kernels), per range in
 // u = T/2^(b + 1) (b: DevMech::th_lo for the low range, 12 for the high one; fx_mul halves): c_p in
 // J/(mol K) (c[0..4]), h in J/mol (c[5..10]: constant, u..u^5) and g in J/mol (c[11..17]: constant,
@@ -150,7 +157,9 @@ struct __align__(16) FxSpecies {
 };
 struct __align__(16) FxEff {
     int64_t w;          // (eps - 1)/W relative to the largest 1/W, units 2^(eff_shift - 62)
-    int32_t sp, slot;   // species, and its slot in the derivative kernels
+    int32_t sp, pad;    // species
+    double wd;          // the same as a double
+    int64_t pad2;
 };
 
 constexpr int kTroeDf = 4;       // float4 records per Troe reaction in DevMech::troe_df
@@ -159,10 +168,27 @@ constexpr int kTroeDf = 4;       // float4 records per Troe reaction in DevMech:
 // of a chunk image and of its pieces, bytes of a species row, and the species in slot order.
 struct FxSet {
     int32_t np, rows, nchunk, image, image_parts, image_spec, image_list, row;
+    int32_t xrows, image_eff, image_effl, pad;        // xrows: most third-body and Troe reactions of a chunk
     const unsigned char* chunks;      // [nchunk][image]
     const FxSpecies* sp;              // [K]
 };
-constexpr int kFxSets = 2;            // 0: rates; 1: derivatives
+// The single-precision products' records and lists: a chunk's image holds FxRxn32 records, the parts'
+// first records (image_parts), one word per species slot (image_spec: start << 8 | count) and the
+// entries (image_list: FxTerm32) in the order in which the sums of k_lin.cu's rounds take them, which
+// fixes their rounding.
+struct __align__(16) FxRxn32 {
+    uint16_t off[8];    // rows (128 bytes per species slot) of the entries: reactants, products from 4
+    int32_t info;       // nr | np << 4 | kind << 8
+    int32_t r, boff;    // device order, first entry slot (DevMech::lin_boff)
+    int32_t eff0, eff1, pad0, pad1, pad2;
+};
+struct FxTerm32 {
+    uint32_t row;       // byte offset of the reaction's row (256 each)
+    float nu;           // signed coefficient
+};
+
+constexpr int kFxSets = 3;            // 0: rates; 1: derivatives; 2: products from stored data (one row of
+                                      // doubles per species)
 
 // Device view of a loaded mechanism (passed by value to every kernel).
 struct DevMech {
@@ -255,13 +281,19 @@ struct DevMech {
     // fixed-point tables of the FP64 reaction kernels (fx_ok: the mechanism fits them)
     int32_t fx_ok, fx_eff_shift;
     FxSet fxs[kFxSets];
+    FxSet fx32[3];                // the single-precision products, summed as by 1, 2, 4 parts' rounds
+    const int32_t* fx32_slot;     // [K] slot of a species in them
     int64_t fx_lmaxw, fx_lR;      // log2(largest 1/W), log2(R)
+    double fx_maxw;               // largest 1/W
     const uint32_t* fx_tab;
     const FxExtra* fx_extra;
+    const int32_t* fx_nu1;        // [R] first reactant's coefficient | first product's << 4 (device order)
     const FxTroe* fx_troe;
     const FxEff* fx_eff;
     // fixed-point thermo polynomials (th_lo: low-range fraction T/2^th_lo; 0: they do not fit)
-    int32_t th_lo, th_pad;
+    int32_t th_lo;
+    int32_t tr_ok;                // the binary diffusion fits in fixed point (128 < T < 4096 K)
+    const int64_t* tr_D;          // [P][4] -log2 D_jk: cubic in log2(T)/32 (fx_mul's halving included)
     const FxThermo* th;
 };
 
@@ -284,7 +316,7 @@ constexpr int kFxOwn = 8;          // species per part of the fixed-point kernel
 // make 32 warps per SM; the derivative kernels 80 registers, 24 warps (6, 2 or 1 blocks: their
 // species rows fill shared memory; 0: they do not fit).
 inline int fx_parts(int K, int set = 0) {
-    if (set == 0) return K <= 4 * kFxOwn ? 4 : K <= 8 * kFxOwn ? 8 : K <= 16 * kFxOwn ? 16 : 32;
+    if (set != 1) return K <= 4 * kFxOwn ? 4 : K <= 8 * kFxOwn ? 8 : K <= 16 * kFxOwn ? 16 : 32;
     return K <= 32 ? 4 : K <= 64 ? 12 : K <= 140 ? 24 : 0;
 }
 }  // namespace nk
