@@ -24,6 +24,7 @@
 #include <utility>
 #include <vector>
 
+#include "k_vjp_fx.cuh"
 #include "nk_rxn.cuh"
 
 namespace nk {
@@ -469,7 +470,8 @@ size_t vjp_smem(int K, int R, int mslots, bool want_g) {
 // PASS 0 takes the tiles of the logarithmic form and skips the others; PASS 1 takes only those
 // (products in double).  Each pass alone compiles to fewer registers than both paths together:
 // the logarithmic pass runs four blocks of 4 warps per SM, the fallback pass three.
-template <int NP, bool WANT_G, bool HB, int PASS>
+// MARKED: only the points whose gT holds kFxSkip (left by k_vjp_fx.cuh, which takes the others).
+template <int NP, bool WANT_G, bool HB, int PASS, bool MARKED = false>
 __global__ void __launch_bounds__(kVjpBlk * NP, (PASS == 0 ? 512 : 384) / (kVjpBlk * NP)) vjp_kernel(const DevMech m, const int64_t n, const int64_t ld,
                                                            const double* __restrict__ T, const double* __restrict__ p,
                                                            const double* __restrict__ Y,
@@ -504,6 +506,11 @@ __global__ void __launch_bounds__(kVjpBlk * NP, (PASS == 0 ? 512 : 384) / (kVjpB
         VjpPoint Q;
         Q.valid = i0 < n;
         const int64_t i = Q.valid ? i0 : n - 1;                   // idle lanes shadow the last point
+        if constexpr (MARKED) {
+            const bool marked = __double_as_longlong(gT[i]) == (long long)kFxSkip;
+            if (__syncthreads_or(marked) == 0) continue;
+            Q.valid &= marked;
+        }
         // logarithmic form unless a point of the tile has a mass fraction outside 2^+-100 (zero,
         // negative, tiny or non-finite): then the products in double (C_k in the row)
         // (and the logarithmic form sums the cotangents bar_omega_k in pairs: each within 2^+-100
@@ -612,12 +619,12 @@ __global__ void reduce_blocks_kernel(const double* __restrict__ ws, int nblocks,
 // ---------------------------------------------------------------- launch plan
 constexpr int kParts[] = {1, 2, 4};
 
-template <bool WANT_G, bool HB, int PASS>
+template <bool WANT_G, bool HB, int PASS, bool MARKED = false>
 const void* kernel_ptr(int c) {
     switch (c) {
-        case 0: return (const void*)vjp_kernel<1, WANT_G, HB, PASS>;
-        case 1: return (const void*)vjp_kernel<2, WANT_G, HB, PASS>;
-        default: return (const void*)vjp_kernel<4, WANT_G, HB, PASS>;
+        case 0: return (const void*)vjp_kernel<1, WANT_G, HB, PASS, MARKED>;
+        case 1: return (const void*)vjp_kernel<2, WANT_G, HB, PASS, MARKED>;
+        default: return (const void*)vjp_kernel<4, WANT_G, HB, PASS, MARKED>;
     }
 }
 
@@ -629,6 +636,7 @@ struct VjpPlan {
     int dev, K, R, ms2, ms4, variant;
     int parts_idx[2];   // index into kParts, per pass
     int grid_cap[2];    // blocks of each pass
+    int fx_cap;         // blocks of the fixed-point kernel (0: it does not take the mechanism)
 };
 std::mutex g_plan_mu;
 std::vector<VjpPlan> g_plans;
@@ -666,7 +674,7 @@ bool plan_variant(const DevMech& m, VjpPlan& out) {
         std::lock_guard<std::mutex> lk(g_plan_mu);
         for (const VjpPlan& q : g_plans)
             if (q.dev == dev && q.K == m.K && q.R == m.R && q.ms2 == m.mslots2 && q.ms4 == m.mslots4 &&
-                q.variant == variant) {
+                q.variant == variant && (q.fx_cap != 0) == vjp_fx_fits(m)) {
                 out = q;
                 return true;
             }
@@ -677,7 +685,13 @@ bool plan_variant(const DevMech& m, VjpPlan& out) {
     int p0 = -1, p1 = -1, b0 = 0, b1 = 0;
     if (!plan_pass<WANT_G, HB, 0>(m, sms, per_block, p0, b0)) return false;
     if (!plan_pass<WANT_G, HB, 1>(m, sms, per_block, p1, b1)) return false;
-    out = VjpPlan{dev, m.K, m.R, m.mslots2, m.mslots4, variant, {p0, p1}, {sms * b0, sms * b1}};
+    out = VjpPlan{dev, m.K, m.R, m.mslots2, m.mslots4, variant, {p0, p1}, {sms * b0, sms * b1}, 0};
+    // with the fixed-point kernel the two passes see only marked points: half a block per SM each,
+    // so that the partial sums' rows stay no more than without it (b0 + b1 blocks per SM)
+    if (vjp_fx_fits(m)) {
+        out.fx_cap = sms * std::min(vjp_fx_blocks(m), std::max(1, b0 + b1 - 1));
+        out.grid_cap[0] = out.grid_cap[1] = std::max(1, sms / 2);
+    }
     std::lock_guard<std::mutex> lk(g_plan_mu);
     g_plans.push_back(out);
     return true;
@@ -693,30 +707,36 @@ int64_t vjp_grid(const VjpPlan& pl, int pass, int64_t n) {
     return tiles < pl.grid_cap[pass] ? tiles : pl.grid_cap[pass];
 }
 
-// blocks of both passes, the ln A partial sums' rows in the workspace
-int64_t vjp_blocks(const VjpPlan& pl, int64_t n) { return vjp_grid(pl, 0, n) + vjp_grid(pl, 1, n); }
+int64_t vjp_fx_grid(const VjpPlan& pl, int64_t n) {
+    const int64_t tiles = (n + kVjpBlk - 1) / kVjpBlk;
+    return tiles < pl.fx_cap ? tiles : pl.fx_cap;
+}
 
-template <bool WANT_G, bool HB, int PASS>
+// blocks of both passes and of the fixed-point kernel before them, the ln A partial sums' rows in
+// the workspace
+int64_t vjp_blocks(const VjpPlan& pl, int64_t n) { return vjp_fx_grid(pl, n) + vjp_grid(pl, 0, n) + vjp_grid(pl, 1, n); }
+
+template <bool WANT_G, bool HB, int PASS, bool MARKED = false>
 cudaError_t launch_pass(const VjpPlan& pl, const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                         const double* Y, const double* dlnA, const double* bar_omega, const double* bar_hrr,
                         double* gT, double* gY, double* ws, cudaStream_t s) {
     const int np = kParts[pl.parts_idx[PASS]];
     const size_t smem = vjp_smem(m.K, m.R, vjp_mslots(m, np), WANT_G);
-    const void* kp = kernel_ptr<WANT_G, HB, PASS>(pl.parts_idx[PASS]);
+    const void* kp = kernel_ptr<WANT_G, HB, PASS, MARKED>(pl.parts_idx[PASS]);
     cudaError_t e = ensure_smem(kp, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)vjp_grid(pl, PASS, n);
     switch (np) {
         case 1:
-            vjp_kernel<1, WANT_G, HB, PASS><<<grid, kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr,
+            vjp_kernel<1, WANT_G, HB, PASS, MARKED><<<grid, kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr,
                                                                         gT, gY, ws);
             break;
         case 2:
-            vjp_kernel<2, WANT_G, HB, PASS><<<grid, 2 * kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega,
+            vjp_kernel<2, WANT_G, HB, PASS, MARKED><<<grid, 2 * kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega,
                                                                             bar_hrr, gT, gY, ws);
             break;
         default:
-            vjp_kernel<4, WANT_G, HB, PASS><<<grid, 4 * kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega,
+            vjp_kernel<4, WANT_G, HB, PASS, MARKED><<<grid, 4 * kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega,
                                                                             bar_hrr, gT, gY, ws);
     }
     return cudaGetLastError();
@@ -726,6 +746,16 @@ template <bool WANT_G, bool HB>
 cudaError_t launch_v(const VjpPlan& pl, const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                      const double* Y, const double* dlnA, const double* bar_omega, const double* bar_hrr, double* gT,
                      double* gY, double* ws, cudaStream_t s) {
+    if (pl.fx_cap) {
+        const int64_t g = vjp_fx_grid(pl, n), g0 = vjp_grid(pl, 0, n);
+        cudaError_t e = launch_vjp_fx<WANT_G, HB>(m, g, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, s);
+        if (e != cudaSuccess) return e;
+        e = launch_pass<WANT_G, HB, 0, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY,
+                                             ws ? ws + (size_t)g * m.R : nullptr, s);
+        if (e != cudaSuccess) return e;
+        return launch_pass<WANT_G, HB, 1, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY,
+                                                ws ? ws + (size_t)(g + g0) * m.R : nullptr, s);
+    }
     cudaError_t e = launch_pass<WANT_G, HB, 0>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, s);
     if (e != cudaSuccess) return e;
     double* ws1 = ws ? ws + (size_t)vjp_grid(pl, 0, n) * m.R : nullptr;
