@@ -37,6 +37,7 @@
 #include <utility>
 #include <vector>
 
+#include "nk_fxpt.cuh"
 #include "nk_lin.cuh"
 
 namespace nk {
@@ -114,7 +115,8 @@ __host__ __device__ constexpr size_t linc_smem(int K, int blk, int np, bool out)
            (size_t)K * blk;
 }
 
-template <int BLK, int NP, bool OUT>
+// MARKED: only the points whose S1 slot holds kFxSkip (left by k_linc_fx.cuh, which takes the others).
+template <int BLK, int NP, bool OUT, bool MARKED = false>
 __global__ void __launch_bounds__(BLK * NP) linc_kernel(const DevMech m, const int64_t n, const int64_t ld,
                                                         const double* __restrict__ T, const double* __restrict__ p,
                                                         const double* __restrict__ Y,
@@ -128,8 +130,13 @@ __global__ void __launch_bounds__(BLK * NP) linc_kernel(const DevMech m, const i
     const int slot = threadIdx.x % BLK, part = threadIdx.x / BLK;
     const int64_t i0 = (int64_t)blockIdx.x * BLK + slot;
     if (NP == 1 && i0 >= n) return;              // (NP = 1 has no barrier below)
-    const bool live = i0 < n;
+    bool live = i0 < n;
     const int64_t i = live ? i0 : n - 1;
+    if constexpr (MARKED) {
+        const bool marked = __double_as_longlong(lin[cs_S(m) * ldl + i]) == (long long)kFxSkip;
+        if (!(NP > 1 ? __syncthreads_or(marked) != 0 : __any_sync(__activemask(), marked))) return;
+        live &= marked;
+    }
     double* sC = smem + kMathTabDoubles + slot;
     double* sW0 = smem + kMathTabDoubles + (size_t)K * BLK + slot;          // OUT: omega_k partials
     double* sW = sW0 + (size_t)part * K * BLK;
@@ -419,6 +426,14 @@ __global__ void __launch_bounds__(BLK * NP) jvpc_kernel(const DevMech m, const i
                                lin + cs_S(m) * ldl + i, ldl, Y, vY, ld, fT, fY, ldf, d_omega, d_hrr);
 }
 
+}  // namespace
+}  // namespace nk
+
+#include "k_linc_fx.cuh"
+
+namespace nk {
+namespace {
+
 // ---------------------------------------------------------------- launch shapes
 struct Shape {
     int blk, np;
@@ -514,6 +529,20 @@ cudaError_t launch_idx(int idx, std::integer_sequence<int, S...>, int K, int64_t
     return e;
 }
 
+// The marked points of the fixed-point pass.
+template <bool OUT>
+cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
+                          const double* dlnA, double* lin, int64_t ldl, double* omega, double* hrr, cudaStream_t s) {
+    int np = m.K >= 8 ? 4 : 1;
+    while (np > 1 && linc_smem(m.K, 32, np, OUT) > smem_limit()) np = 1;
+    const size_t smem = linc_smem(m.K, 32, np, OUT);
+    auto kern = np == 4 ? linc_kernel<32, 4, OUT, true> : linc_kernel<32, 1, OUT, true>;
+    const cudaError_t e = ensure_smem((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((n + 31) / 32), 32 * np, smem, s>>>(m, n, ld, T, p, Y, dlnA, lin, ldl, omega, hrr);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 int64_t linc_slots(const DevMech& m) { return cs_C(m) + m.K; }
@@ -522,6 +551,13 @@ cudaError_t launch_linearize_compact(const DevMech& m, int64_t n, int64_t ld, co
                                      const double* Y, const double* dlnA, double* lin, int64_t ldl, double* omega,
                                      double* hrr, cudaStream_t s) {
     static_assert(kDfTabBytes <= kMathTabDoubles * sizeof(double), "table space");
+    if (linc_fx_fits(m)) {
+        cudaError_t e = omega ? launch_linc_fx<true>(m, n, ld, T, p, Y, dlnA, lin, ldl, omega, hrr, s)
+                              : launch_linc_fx<false>(m, n, ld, T, p, Y, dlnA, lin, ldl, omega, hrr, s);
+        if (e != cudaSuccess) return e;
+        return omega ? launch_marked<true>(m, n, ld, T, p, Y, dlnA, lin, ldl, omega, hrr, s)
+                     : launch_marked<false>(m, n, ld, T, p, Y, dlnA, lin, ldl, omega, hrr, s);
+    }
     if (omega) {
         const int idx = plan_shape<1>(m.K);
         if (idx < 0) return cudaErrorInvalidConfiguration;
@@ -539,6 +575,9 @@ cudaError_t launch_jvp_linearized_compact(const DevMech& m, int64_t n, int64_t l
                                           const double* Y, const double* lin, int64_t ldl, const double* fT,
                                           const double* fY, int64_t ldf, const double* vT, const double* vY,
                                           double* d_T, double* d_Y, cudaStream_t s, int rhs) {
+    if (m.fx_ok && m.K >= 3 && jvpc_fx_smem(m) <= smem_limit())
+        return rhs ? launch_jvpc_fx<true>(m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, fT, fY, ldf, s)
+                   : launch_jvpc_fx<false>(m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, nullptr, nullptr, 0, s);
     if (rhs) {
         const int idx = plan_shape<3>(m.K);
         if (idx < 0) return cudaErrorInvalidConfiguration;

@@ -262,33 +262,22 @@ __device__ __forceinline__ FxRate fx_sides(const unsigned char* sp, int info, ui
 static __device__ __noinline__ double fx_shift_edge(double q, double d) { return q * exp(d); }
 
 // Sum over one species' rows of a chunk, the rows MUL 256 bytes apart (w: its word in the image,
-// list: the image's row list, q: the rows, this lane's column), added to s in list order.  Two rows
-// are loaded at a time (the chain of additions stays one).
-template <int MUL>
-__device__ __forceinline__ double fx_row(const unsigned char* q, const unsigned char* l) {
-    return *reinterpret_cast<const double*>(q + MUL * *reinterpret_cast<const uint16_t*>(l));
-}
+// list: the image's row list, q: the rows, this lane's column), added to s in list order.  (Two rows
+// per step left predicated FP64 additions behind, which cost as much as executed ones.)
 template <int MUL = 1>
 __device__ __forceinline__ double fx_gather(uint32_t w, const unsigned char* list, const unsigned char* q, double s) {
     const unsigned char* l = list + (w >> 15 & ~1u);
     const unsigned char* e = l + (w >> 7 & 510u);
 #pragma unroll 1
-    for (; e - l >= 4; l += 4) {
-        const double a = fx_row<MUL>(q, l), b = fx_row<MUL>(q, l + 2);
-        s += a;
-        s += b;
-    }
-    if (l != e) s += fx_row<MUL>(q, l);
-    l = e;
+    for (; l != e; l += 2) s += *reinterpret_cast<const double*>(q + MUL * *reinterpret_cast<const uint16_t*>(l));
     e += (w & 255u) * 2;
 #pragma unroll 1
-    for (; e - l >= 4; l += 4) {
-        const double a = fx_row<MUL>(q, l), b = fx_row<MUL>(q, l + 2);
-        s -= a;
-        s -= b;
-    }
-    if (l != e) s -= fx_row<MUL>(q, l);
+    for (; l != e; l += 2) s -= *reinterpret_cast<const double*>(q + MUL * *reinterpret_cast<const uint16_t*>(l));
     return s;
 }
+
+// q times a stoichiometric coefficient other than 1.  Out of line: inline it becomes a predicated
+// conversion and product on the FP64 pipe for every reaction.
+static __device__ __noinline__ double times_nu(double q, int nu) { return q * (double)nu; }
 
 }  // namespace nk
