@@ -107,7 +107,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             }
         }
         const bool valid = live && good;
-        const double hbRT = HB ? bar_hrr[i] * (kR * Ti) : 0.0;
+        const double hbRT = HB ? bar_hrr[i] * (kR * Ti) : 0.0, hbCp = -hbRT * kFxCpScale;
         fx_image_wait();
         __syncthreads();
 
@@ -170,7 +170,6 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                 }
                 long long z = 1;
                 dfl px{1.0f, 0.0f};
-                dfl st{0.0f, 0.0f};                      // Troe: T d ln F/dT
                 const int kind = info >> 8 & 3;
                 if (kind != 0) {
                     const int4 x = __ldg(reinterpret_cast<const int4*>(m.fx_extra + (info >> 16)));
@@ -188,7 +187,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                         lnk += t.phi;
                         const long long s0 = (a.y >> 5) - fx_scale(e0, 0x58B90BFBE8E7BCD6ull);
                         px = t.px;
-                        st = df_fma(px, fx_to_pair(s0 - s), t.pt);
+                        s += fx_of_pair(df_fma(px, fx_to_pair(s0 - s), t.pt));   // with T d ln F/dT
                     }
                 }
                 if (kind != 1) lnk &= ~1ll;
@@ -203,11 +202,9 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                 if (!valid) qf = qr = 0.0;
                 const double F = qbar * qf, B = -qbar * qr;
                 const double G = F + B;
-                double sd = fx_to_d(s);
-                if (kind == 2) sd += df_to_d(st);
-                Tbar = fma(G, sd, Tbar);
+                Tbar = fma(G, fx_to_d(s), Tbar);
                 Tbar = fma(B, fx_to_d(E), Tbar);
-                if constexpr (HB) Tbar = fma(-hbRT * kFxCpScale * (qf - qr), fx_to_d(Cp), Tbar);
+                if constexpr (HB) Tbar = fma(hbCp * (qf - qr), fx_to_d(Cp), Tbar);
                 if (kind != 0) {
                     // X = G px rho'/[M] (z in units 2^(eff_shift - 60)); the p/(RT) part of [M]
                     double X = 0.0;
@@ -253,18 +250,21 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                 }
             }
             if (WANT_G) {
-                // lane l of warp g sums row 32 g + l over the points, starting at its own column (no
-                // two lanes in one bank)
-                const int rows = im[f.image_parts + NP];
-                for (int row = part * 32 + lane; row < rows; row += NP * 32) {
+                // four lanes sum a row over the points, eight columns each (the rows, 512 bytes apart, start
+                // at different columns: two lanes a bank at most), then over the four
+                const int rows = im[f.image_parts + NP], g = lane >> 2, h = lane & 3;
+                for (int r8 = part * 8; r8 < rows; r8 += NP * 8) {
+                    const int row = min(r8 + g, rows - 1);
                     const double* q = reinterpret_cast<const double*>(sQ - lane * 8 + row * 512);
                     double a = 0.0;
 #pragma unroll 4
-                    for (int c2 = 0; c2 < 32; ++c2) {
-                        const int col = (c2 + lane) & 31;
+                    for (int c2 = 0; c2 < 8; ++c2) {
+                        const int col = h * 8 + ((c2 + g) & 7);
                         a += q[col] + q[32 + col];
                     }
-                    gw[reinterpret_cast<const FxRxn*>(im)[row].orig >> 16] += a;
+                    a += __shfl_xor_sync(0xffffffffu, a, 1);
+                    a += __shfl_xor_sync(0xffffffffu, a, 2);
+                    if (h == 0 && r8 + g < rows) gw[reinterpret_cast<const FxRxn*>(im)[row].orig >> 16] += a;
                 }
             }
             fx_image_wait();
