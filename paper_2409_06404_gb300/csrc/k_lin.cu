@@ -137,6 +137,14 @@ __device__ __forceinline__ void store_coef(const DevMech& m, int r, float* lin, 
     }
 }
 
+}  // namespace
+}  // namespace nk
+
+#include "k_lin_fx.cuh"
+
+namespace nk {
+namespace {
+
 // ---------------------------------------------------------------- linearization pass
 template <int BLK, int KIND, class TS>
 __device__ __forceinline__ void lin_reaction(const DevMech& m, int r, const double* sC, const LinPoint& Q,
@@ -206,8 +214,9 @@ __device__ __forceinline__ void lin_group(const DevMech& m, int r0, int r1, cons
     for (int r = r0; r < r1; ++r) lin_reaction<BLK, KIND>(m, r, sC, Q, dlnA, dt, lin, ldl, i, live, S1, sE);
 }
 
-// TS: the stored type (double, or float for the single-precision products)
-template <int BLK, int NP, class TS>
+// TS: the stored type (double, or float for the single-precision products).  MARKED: only the points
+// whose S1 slot holds kFxSkip (left by k_lin_fx.cuh, which takes the others).
+template <int BLK, int NP, class TS, bool MARKED = false>
 __global__ void __launch_bounds__(BLK * NP, 512 / (BLK * NP)) linearize_kernel(const DevMech m, const int64_t n, const int64_t ld,
                                                              const double* __restrict__ T,
                                                              const double* __restrict__ p,
@@ -222,8 +231,13 @@ __global__ void __launch_bounds__(BLK * NP, 512 / (BLK * NP)) linearize_kernel(c
     const int slot = threadIdx.x % BLK, part = threadIdx.x / BLK;
     const int64_t i0 = (int64_t)blockIdx.x * BLK + slot;
     if (NP == 1 && i0 >= n) return;              // (NP = 1 has no barrier below)
-    const bool live = i0 < n;
+    bool live = i0 < n;
     const int64_t i = live ? i0 : n - 1;
+    if constexpr (MARKED) {
+        const bool marked = get_s1(lin, slot_S(m) * ldl + i, ldl) == kFxSkip;
+        if (!(NP > 1 ? __syncthreads_or(marked) != 0 : __any_sync(__activemask(), marked))) return;
+        live &= marked;
+    }
     double* sC = smem + kMathTabDoubles + slot;
     // float format: the species' exponent scales E_k (K ints per point after C_k)
     int* sE = F32 ? reinterpret_cast<int*>(smem + kMathTabDoubles + (size_t)K * BLK) + slot : nullptr;
@@ -581,6 +595,14 @@ __device__ __forceinline__ void apply_rounds32(const DevMech& m, int part, const
         [&](int, const RxnLin32& v) { apply_one32<BLK, KIND>(m, v.x, v.c, sdC, sD, sE, tT, dpRT); });
 }
 
+}  // namespace
+}  // namespace nk
+
+#include "k_lin32_fx.cuh"
+
+namespace nk {
+namespace {
+
 // Shared memory: 3 NP sums per point (double), the row of scaled d omega_k sums, dC_k, E_k
 // (4-byte words).
 __host__ __device__ constexpr size_t lin32_smem(int K, int blk, int np) {
@@ -803,6 +825,21 @@ cudaError_t launch_idx(int idx, std::integer_sequence<int, S...>, int K, int64_t
     return e;
 }
 
+// The linearization: the fixed-point pass and its marked points, where the mechanism fits.
+template <class TS>
+cudaError_t launch_lin_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
+                              const double* dlnA, TS* lin, int64_t ldl, cudaStream_t s) {
+    cudaError_t e = launch_lin_fx(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
+    if (e != cudaSuccess) return e;
+    const Shape sh{32, m.K >= 8 ? 4 : 1};
+    const size_t smem = lin_smem(m.K, sh, sizeof(TS) == sizeof(float) ? 5 : 0);
+    auto kern = sh.np == 4 ? linearize_kernel<32, 4, TS, true> : linearize_kernel<32, 1, TS, true>;
+    e = ensure_smem((const void*)kern, smem);
+    if (e != cudaSuccess) return e;
+    kern<<<(unsigned)((n + 31) / 32), 32 * sh.np, smem, s>>>(m, n, ld, T, p, Y, dlnA, lin, ldl);
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 int64_t lin_slots(const DevMech& m) { return slot_H(m) + m.K; }
@@ -811,6 +848,7 @@ int64_t lin_slots_f32(const DevMech& m) { return slot_EK32(m) + m.K; }
 cudaError_t launch_linearize(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                              const double* Y, const double* dlnA, double* lin, int64_t ldl, cudaStream_t s) {
     static_assert(kDfTabBytes <= kMathTabDoubles * sizeof(double), "table space");
+    if (lin_fx_fits(m)) return launch_lin_marked(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
     const int idx = plan_shape<0>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
     return launch_idx<0>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, dlnA,
@@ -829,6 +867,7 @@ cudaError_t launch_jvp_linearized(const DevMech& m, int64_t n, int64_t ld, const
 
 cudaError_t launch_linearize_f32(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                                  const double* Y, const double* dlnA, float* lin, int64_t ldl, cudaStream_t s) {
+    if (lin_fx_fits(m)) return launch_lin_marked(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
     const int idx = plan_shape<5>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
     return launch_idx<5>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, dlnA,
@@ -842,11 +881,15 @@ cudaError_t launch_jvp_linearized_f32(const DevMech& m, int64_t n, int64_t ld, c
     if (rhs) {
         const int idx = plan_shape<4>(m.K);
         if (idx < 0) return cudaErrorInvalidConfiguration;
+        if (m.fx_ok)
+            return launch_lin32_fx<true>(kShapes[idx].np, m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, fT, fY, ldf, s);
         return launch_idx<4>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, lin,
                              ldl, vT, vY, d_Y, d_T, fT, fY, ldf);
     }
     const int idx = plan_shape<3>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
+    if (m.fx_ok)
+        return launch_lin32_fx<false>(kShapes[idx].np, m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, nullptr, nullptr, 0, s);
     const double* none = nullptr;
     return launch_idx<3>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, lin, ldl,
                          vT, vY, d_Y, d_T, none, none, (int64_t)0);
