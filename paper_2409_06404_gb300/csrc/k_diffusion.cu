@@ -5,26 +5,26 @@
 // With Y_k/X_k = W_k/Wbar the uncorrected flux rho Y_k V'_k = a_k grad X_k,
 // a_k = -rho (W_k/Wbar) D_k, has no division by X_k; with S = sum_k a_k grad X_k,
 // V_c = -S/rho and j_k = a_k grad X_k - Y_k S.  One thread per point, two passes over the
-// species (the second re-reads grad X_k, which the first brought into L2, and takes a_k from
-// shared memory); the pass reads 3K + 2K + 2 and writes 3K + 6 doubles per point.  The FP64 pipe
-// bounds it: 14 operations per species and point; c_p,k comes from integer polynomials
-// (nk_thermo.cuh) for 64 K <= T < 4096 K, with them and a_k formed again it took 23.
+// species (the second re-reads D_k and grad X_k, which the first brought into L2); the pass reads
+// 3K + 2K + 2 and writes 3K + 6 doubles per point.  The FP64 pipe bounds it: 15 operations per
+// species and point; c_p,k comes from integer polynomials (nk_thermo.cuh) for 64 K <= T < 4096 K,
+// with it in doubles it took 23.  (Keeping a_k in shared memory between the passes saves one more
+// but holds the SM at 16 warps.)  With the thermodynamics, 53 species, 884,736 points: 4.05 -> 2.12 ms
+// (3.09 with 64 threads and the shared array).
 #include "nk_thermo.cuh"
 
 namespace nk {
 namespace {
 
-constexpr int kBlk = 64;
+constexpr int kBlk = 128;
 
 __global__ void __launch_bounds__(kBlk) diffusion_kernel(const DevMech m, const int64_t n, const int64_t ld,
                                                          const double* __restrict__ T, const double* __restrict__ p,
                                                          const double* __restrict__ Y, const double* __restrict__ D,
                                                          const double* __restrict__ G, double* __restrict__ j,
                                                          double* __restrict__ Vc, double* __restrict__ hf) {
-    extern __shared__ double sm[];
     const int64_t i = (int64_t)blockIdx.x * kBlk + threadIdx.x;
     if (i >= n) return;
-    double* sa = sm + threadIdx.x;                            // a_k / c0 = W_k D_k at sa[k kBlk]
     const int K = m.K;
     const int64_t cs = (int64_t)K * ld;                       // component stride of grad X and j
     const double Ti = T[i];
@@ -32,8 +32,7 @@ __global__ void __launch_bounds__(kBlk) diffusion_kernel(const DevMech m, const 
     for (int k = 0; k < K; ++k) {
         const int64_t o = (int64_t)k * ld + i;
         s = fma(Y[o], __ldg(m.invW + k), s);
-        const double a = __ldg(m.W + k) * D[o];
-        sa[k * kBlk] = a;
+        const double a = __ldg(m.W + k) * D[o];               // a_k / c0
         S0 = fma(a, G[o], S0);
         S1 = fma(a, G[o + cs], S1);
         S2 = fma(a, G[o + 2 * cs], S2);
@@ -53,7 +52,7 @@ __global__ void __launch_bounds__(kBlk) diffusion_kernel(const DevMech m, const 
     double h0 = 0.0, h1 = 0.0, h2 = 0.0;
     for (int k = 0; k < K; ++k) {
         const int64_t o = (int64_t)k * ld + i;
-        const double a = c0 * sa[k * kBlk], y = Y[o];
+        const double a = c0 * (__ldg(m.W + k) * D[o]), y = Y[o];
         const double j0 = fma(a, G[o], -y * S0), j1 = fma(a, G[o + cs], -y * S1), j2 = fma(a, G[o + 2 * cs], -y * S2);
         j[o] = j0;
         j[o + cs] = j1;
@@ -85,10 +84,7 @@ __global__ void __launch_bounds__(kBlk) diffusion_kernel(const DevMech m, const 
 cudaError_t launch_diffusion(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                              const double* Y, const double* D, const double* gradX, double* j, double* Vc,
                              double* hf, cudaStream_t s) {
-    const size_t smem = (size_t)m.K * kBlk * sizeof(double);
-    const cudaError_t e = ensure_smem((const void*)diffusion_kernel, smem);
-    if (e != cudaSuccess) return e;
-    diffusion_kernel<<<(unsigned)((n + kBlk - 1) / kBlk), kBlk, smem, s>>>(m, n, ld, T, p, Y, D, gradX, j, Vc, hf);
+    diffusion_kernel<<<(unsigned)((n + kBlk - 1) / kBlk), kBlk, 0, s>>>(m, n, ld, T, p, Y, D, gradX, j, Vc, hf);
     return cudaGetLastError();
 }
 
