@@ -16,11 +16,15 @@ cudaError_t launch_rates(const DevMech& m, int64_t n, int64_t ld, const double* 
     // the staged tables (kMathTabDoubles doubles) cover the kDF tables too (3 x 128 pairs)
     static_assert(kDfTabBytes <= kMathTabDoubles * sizeof(double), "table space");
     if (rhs) return launch_rates_rhs(m, n, ld, T, p, Y, dlnA, omega, hrr, precision, s);
+    if (precision == NK_MIXED && m.fx_ok) {
+        const cudaError_t e = launch_rates_fx<false, true>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+        return e != cudaSuccess ? e : launch_marked<kMixed, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+    }
     if (precision == NK_MIXED) return launch_form<kMixed, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
     if (precision == NK_FP64_NATIVE) return launch_form<kNative, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
     if (m.fx_ok) {
-        const cudaError_t e = launch_rates_fx<false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
-        return e != cudaSuccess ? e : launch_marked<false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+        const cudaError_t e = launch_rates_fx<false, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
+        return e != cudaSuccess ? e : launch_marked<kDF, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
     }
     return launch_form<kDF, false>(m, n, ld, T, p, Y, dlnA, omega, hrr, s);
 }

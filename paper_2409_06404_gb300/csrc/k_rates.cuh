@@ -359,7 +359,7 @@ __host__ __device__ constexpr int shared_rows() {
 //
 // RHS: write the implicit-stage sources instead: omega -> W_k omega_k / rho, hrr -> hrr/(rho c_p).
 //
-// PASS 2 (kDF): as 1 for the points whose hrr holds kFxSkip, whatever their state.  PASS (kDF and kMixed): 0 takes the blocks without a negative concentration and skips the
+// PASS 2 (kDF, kMixed): as 1 for the points whose hrr holds kFxSkip, whatever their state.  PASS (kDF and kMixed): 0 takes the blocks without a negative concentration and skips the
 // others, 1 takes only those, with the concentrations' signs in a byte row after the omega_k row
 // (rates_smem_signs); so the common pass carries no sign work.  The second pass leaves at once
 // where no mass fraction of the block is negative.  The native form has one pass (0) over every
@@ -556,14 +556,14 @@ cudaError_t launch_idx(int idx, std::integer_sequence<int, S...>, const DevMech&
 }
 
 
-// The points that the fixed-point kernel (k_rates_fx.cuh) left marked in hrr, in the kDF form with
-// signs (any state).
-template <bool RHS>
+// The points that the fixed-point kernel (k_rates_fx.cuh) left marked in hrr, in the kDF or
+// kMixed form with signs (any state).
+template <int PREC, bool RHS>
 cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
                           const double* dlnA, double* omega, double* hrr, cudaStream_t st) {
     const Shape sh{32, m.K >= 8 ? 4 : 1};
-    const size_t smem = rates_smem<kDF>(m.K, sh) + rates_smem_signs(m.K, sh);
-    auto kern = sh.np == 4 ? rates_kernel<32, 4, kDF, RHS, 2> : rates_kernel<32, 1, kDF, RHS, 2>;
+    const size_t smem = rates_smem<PREC>(m.K, sh) + rates_smem_signs(m.K, sh);
+    auto kern = sh.np == 4 ? rates_kernel<32, 4, PREC, RHS, 2> : rates_kernel<32, 1, PREC, RHS, 2>;
     const cudaError_t e = ensure_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)((n + 31) / 32), 32 * sh.np, smem, st>>>(m, n, ld, T, p, Y, dlnA, omega, hrr);

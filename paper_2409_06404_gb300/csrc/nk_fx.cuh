@@ -234,4 +234,15 @@ __device__ __forceinline__ long long fx_log2e_times(double d) {
     return v + fx_mul(v, FxFrac{(int32_t)((F + 0x80000000ull) >> 32), (int32_t)(uint32_t)F});
 }
 
+// a float of magnitude below 4096 times log2(e), as fx
+__device__ __forceinline__ long long fx_log2e_times(float f) {
+    const uint32_t b = __float_as_uint(f);
+    const int sh = (int)(b >> 23 & 0xffu) - 127 + kFxS - 23;                          // m 2^sh units
+    const long long m = (long long)((b & 0x7fffffu) | 0x800000u);
+    long long v = sh >= 0 ? m << (sh & 63) : (sh > -24 ? m >> -sh : 0);
+    if ((int)b < 0) v = -v;
+    constexpr unsigned long long F = 0x71547652B82FE177ull;                           // 0.88539008177792681... 2^63
+    return v + fx_mul(v, FxFrac{(int32_t)((F + 0x80000000ull) >> 32), (int32_t)(uint32_t)F});
+}
+
 }  // namespace nk

@@ -80,8 +80,8 @@ __device__ __forceinline__ const int64_t* fx_range(const FxSpecies* s, double T)
 
 // Shared memory of a block (after the fixed-point and the pair tables): the scalars of its points, log2 C_k, mu_k and the
 // rates of progress of one chunk, each as rows of 32 lanes.
-constexpr int kFxScalars = 5;      // log2 T, 128/T (63 bits), log2(p/(R T)), log2 rho', sum Y/W
-enum { kFxLT = 0, kFxV = 1, kFxLpRT = 2, kFxLrho = 3, kFxSum = 4 };
+constexpr int kFxScalars = 6;      // log2 T, 128/T (63 bits), log2(p/(R T)), log2 rho', sum Y/W, floats of ln T and 1/T
+enum { kFxLT = 0, kFxV = 1, kFxLpRT = 2, kFxLrho = 3, kFxSum = 4, kFxTf = 5 };
 constexpr size_t kFxBase = kFxTabBytes + kDfTabBytes;
 // The row after the last species is zero; two chunk images are double buffered; row_bytes per
 // reaction of a chunk.
