@@ -103,7 +103,7 @@ __device__ __forceinline__ void fx_image_load(const FxSet& f, int c, unsigned ch
 __device__ __forceinline__ void fx_image_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---- the state a point needs for the fixed-point form, and its scalars
-constexpr unsigned long long kFxPoison = 1ull << 60;
+constexpr unsigned long long kFxPoison = 1ull << 55;      // (added by up to 32 parts without wrapping)
 __device__ __forceinline__ bool fx_T_ok(double T) {      // 128 (1 + 2^-31) < T < 4096 (1 - 2^-30)
     const long long b = __double_as_longlong(T);
     return b > 0x4060000000200000ll && b < 0x40afffffffc00000ll;
