@@ -3,7 +3,11 @@
 // the others, so all its warps' loads are in flight at once, where the rounds of jvp_lin32_kernel
 // let one reaction per warp load between barriers (1.7 TB/s of the stored words at 2,097,152
 // points).  A species' terms are summed in the order of those rounds (FxTerm32) and the point sums
-// by the same parts, so the results are the same bits.
+// by the same parts, so the results are the same bits.  Load latency bounds it (waits on stored words
+// 4.2 cycles per issue, issue slots 51% busy), so a reaction's words are loaded while the one before
+// is summed, and all parts load the state.  53 species, 65,536 points: 0.38 ms per product (1.7 TB/s
+// of the stored words); the single-precision stage of 175,616 points,
+// with its ten products: 21.9 -> 15.8 ms.
 #pragma once
 
 #include "nk_fxpt.cuh"
@@ -13,6 +17,30 @@ namespace {
 
 inline size_t lin32_fx_smem(const FxSet& f, int K, int old_np) {
     return (size_t)3 * old_np * 256 + 5 * 128 + 128 + 2 * (size_t)f.image + (size_t)K * 384 + (size_t)f.rows * 256;
+}
+inline const FxSet& lin32_set(const DevMech& m, int old_np) { return m.fx32[old_np == 1 ? 0 : old_np == 2 ? 1 : 2]; }
+inline bool lin32_fx_fits(const DevMech& m, int old_np) {
+    return m.fx_ok && lin32_fx_smem(lin32_set(m, old_np), m.K, old_np) <= smem_limit();
+}
+
+// the stored words of one reaction
+struct Words32 {
+    float A, br[kMaxSide], bp[kMaxSide], L;
+    int er;
+};
+__device__ __forceinline__ void load_words32(const DevMech& m, const unsigned char* im, int q, const float* a, int64_t ldl,
+                                             Words32& w) {
+    const int4 h = reinterpret_cast<const int4*>(im + q * (int)sizeof(FxRxn32))[1];      // info, r, boff, eff0
+    const int nr = h.x & 15, np = h.x >> 4 & 15;
+    w.A = __ldcs(a + (int64_t)h.y * ldl);
+    const float* B = a + ((int64_t)m.R + h.z) * ldl;
+#pragma unroll
+    for (int e = 0; e < kMaxSide; ++e) {
+        w.br[e] = e < nr ? __ldcs(B + (int64_t)e * ldl) : 0.0f;
+        w.bp[e] = e < np ? __ldcs(B + (int64_t)(nr + e) * ldl) : 0.0f;
+    }
+    w.er = __ldcs(reinterpret_cast<const int32_t*>(a) + (slot_E32(m) + h.y) * ldl);
+    w.L = h.x >> 8 != 0 ? __ldcs(a + (slot_M(m) + (h.y - m.R_el)) * ldl) : 0.0f;
 }
 
 // OLD: the parts of jvp_lin32_kernel's shape for this mechanism.
@@ -39,6 +67,13 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
     int* sE = reinterpret_cast<int*>(sW + (size_t)K * 32);                       // E_k, species order
     unsigned char* sQ = reinterpret_cast<unsigned char*>(sE + (size_t)K * 32) + lane * 4;   // dq and exponent, 8 bytes a lane
     const int32_t* linE = reinterpret_cast<const int32_t*>(lin) + slot_EK32(m) * ldl + i;
+    // (Y and vY go through the rows of the sums and of E_k, so that all parts load; summed in species order)
+#pragma unroll 4
+    for (int k = part; k < K; k += NP) {
+        sW[k * 32] = narrow(Y[(int64_t)k * ld + i]);
+        sE[k * 32] = __float_as_int(narrow(vY[(int64_t)k * ld + i]));
+    }
+    __syncthreads();
     if (part == 0) {
         const float Ti = narrow(T[i]), dT = narrow(vT[i]);
         const float invT = 1.0f / Ti, tT = dT * invT;
@@ -47,8 +82,8 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
 #pragma unroll 4
         for (int k = 0; k < K; ++k) {
             const float iw = __ldg(m.f_invW + k);
-            s = fmaf(narrow(Y[(int64_t)k * ld + i]), iw, s);
-            ds = fmaf(narrow(vY[(int64_t)k * ld + i]), iw, ds);
+            s = fmaf(sW[k * 32], iw, s);
+            ds = fmaf(__int_as_float(sE[k * 32]), iw, ds);
         }
         const float rho = pRT / s;
         sV[0] = tT;
@@ -59,12 +94,13 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
     __syncthreads();
     {
         const float rho = sV[32], arho = sV[64];
-#pragma unroll 1
+#pragma unroll 4
         for (int k = part; k < K; k += NP) {
             const float iw = __ldg(m.f_invW + k);
+            const int ek = linE[(int64_t)k * ldl];
             *reinterpret_cast<float*>(sdC + (size_t)__ldg(m.fx32_slot + k) * 128) =
-                fmaf(narrow(Y[(int64_t)k * ld + i]) * iw * rho, arho, rho * narrow(vY[(int64_t)k * ld + i]) * iw);
-            sE[k * 32] = linE[(int64_t)k * ldl];
+                fmaf(sW[k * 32] * iw * rho, arho, rho * __int_as_float(sE[k * 32]) * iw);
+            sE[k * 32] = ek;
         }
     }
     fx_image_wait();
@@ -77,8 +113,13 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
         w[j] = 0.0f;
         ek[j] = part + NP * j < K ? sE[__ldg(&f.sp[part + NP * j].k) * 32] : 0;
     }
+    // each part's next reaction is loaded while this one is summed, also across the chunks
+    const float* a = lin + i;
+    Words32 x;
+    if (im0[f.image_parts + part] < im0[f.image_parts + part + 1]) load_words32(m, im0, im0[f.image_parts + part], a, ldl, x);
     for (int c = 0; c < f.nchunk; ++c) {
         const unsigned char* im = im0 + (c & 1) * f.image;
+        const unsigned char* in = im0 + ((c + 1) & 1) * f.image;
         fx_image_load(f, c + 1, im0 + ((c + 1) & 1) * f.image);
         const int q1 = im[f.image_parts + part + 1];
 #pragma unroll 1
@@ -86,37 +127,31 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
             const int4* rec = reinterpret_cast<const int4*>(im + q * (int)sizeof(FxRxn32));
             const int4 o4 = rec[0], h = rec[1];                  // offsets; info, r, boff, eff0
             const int nr = h.x & 15, np = h.x >> 4 & 15, kind = h.x >> 8;
-            const float* a = lin + i;
-            const float A = __ldcs(a + (int64_t)h.y * ldl);
-            const float* B = a + ((int64_t)m.R + h.z) * ldl;
-            float br[kMaxSide], bp[kMaxSide];
-#pragma unroll
-            for (int e = 0; e < kMaxSide; ++e) {
-                br[e] = e < nr ? __ldcs(B + (int64_t)e * ldl) : 0.0f;
-                bp[e] = e < np ? __ldcs(B + (int64_t)(nr + e) * ldl) : 0.0f;
-            }
-            const int er = __ldcs(reinterpret_cast<const int32_t*>(a) + (slot_E32(m) + h.y) * ldl);
-            const float Lc = kind != 0 ? __ldcs(a + (slot_M(m) + (h.y - m.R_el)) * ldl) : 0.0f;
+            const Words32 v = x;
+            if (q + 1 < q1) load_words32(m, im, q + 1, a, ldl, x);
             const unsigned of[8] = {(unsigned)o4.x & 0xffffu, (unsigned)o4.x >> 16, (unsigned)o4.y & 0xffffu, (unsigned)o4.y >> 16,
                                     (unsigned)o4.z & 0xffffu, (unsigned)o4.z >> 16, (unsigned)o4.w & 0xffffu, (unsigned)o4.w >> 16};
-            float dq = A * sV[0];
+            float dq = v.A * sV[0];
 #pragma unroll
             for (int e = 0; e < kMaxSide; ++e)
-                if (e < nr) dq = fmaf(br[e], *reinterpret_cast<const float*>(sdC + of[e]), dq);
+                if (e < nr) dq = fmaf(v.br[e], *reinterpret_cast<const float*>(sdC + of[e]), dq);
 #pragma unroll
             for (int e = 0; e < kMaxSide; ++e)
-                if (e < np) dq = fmaf(bp[e], *reinterpret_cast<const float*>(sdC + of[4 + e]), dq);
+                if (e < np) dq = fmaf(v.bp[e], *reinterpret_cast<const float*>(sdC + of[4 + e]), dq);
             if (kind != 0) {
                 float dM = sV[96];
                 const int e1 = rec[2].x;
                 for (int j = h.w; j < e1; ++j)
                     dM = fmaf(__ldg(m.f_eff_m1 + j),
                               *reinterpret_cast<const float*>(sdC + (size_t)__ldg(m.fx32_slot + __ldg(m.eff_sp + j)) * 128), dM);
-                dq = fmaf(Lc, dM, dq);
+                dq = fmaf(v.L, dM, dq);
             }
-            *reinterpret_cast<int2*>(sQ + q * 256) = make_int2(__float_as_int(dq), er);
+            *reinterpret_cast<int2*>(sQ + q * 256) = make_int2(__float_as_int(dq), v.er);
         }
+        fx_image_wait();
         __syncthreads();
+        if (c + 1 < f.nchunk && in[f.image_parts + part] < in[f.image_parts + part + 1])
+            load_words32(m, in, in[f.image_parts + part], a, ldl, x);
         const uint32_t* spec = reinterpret_cast<const uint32_t*>(im + f.image_spec);
 #pragma unroll
         for (int j = 0; j < kFxOwn; ++j)
@@ -132,7 +167,6 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
                 }
                 w[j] = acc;
             }
-        fx_image_wait();
         __syncthreads();
     }
 #pragma unroll
@@ -148,6 +182,7 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
     float cpm = 0.0f, dcpm = 0.0f;
     const float inv_rho = RHS ? 1.0f / rho : 0.0f;
     const double arho_d = widen(arho);
+#pragma unroll 2
     for (int k = part; k < K; k += OLD) {
         double dw = scale2(widen(sW[k * 32]), sE[k * 32]);
         hsum = fma(widen(lin[(slot_H32(m) + k) * ldl + i]), dw, hsum);
@@ -203,7 +238,7 @@ template <int OLD, bool RHS>
 cudaError_t launch_lin32_fx(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
                             const float* lin, int64_t ldl, const double* vT, const double* vY, double* d_omega,
                             double* d_hrr, const double* fT, const double* fY, int64_t ldf, cudaStream_t s) {
-    const FxSet& f = m.fx32[OLD == 1 ? 0 : OLD == 2 ? 1 : 2];
+    const FxSet& f = lin32_set(m, OLD);
     const size_t smem = lin32_fx_smem(f, m.K, OLD);
     auto kern = f.np == 4 ? jvp_lin32_fx_kernel<4, OLD, RHS> : f.np == 8 ? jvp_lin32_fx_kernel<8, OLD, RHS>
               : f.np == 16 ? jvp_lin32_fx_kernel<16, OLD, RHS> : jvp_lin32_fx_kernel<32, OLD, RHS>;
