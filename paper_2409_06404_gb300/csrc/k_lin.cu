@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(BLK * NP, 512 / (BLK * NP)) linearize_kernel(c
     bool live = i0 < n;
     const int64_t i = live ? i0 : n - 1;
     if constexpr (MARKED) {
-        const bool marked = get_s1(lin, slot_S(m) * ldl + i, ldl) == kFxSkip;
+        const bool marked = __double_as_longlong(lin[slot_S(m) * ldl + i]) == (long long)kFxSkip;
         if (!(NP > 1 ? __syncthreads_or(marked) != 0 : __any_sync(__activemask(), marked))) return;
         live &= marked;
     }
@@ -826,14 +826,13 @@ cudaError_t launch_idx(int idx, std::integer_sequence<int, S...>, int K, int64_t
 }
 
 // The linearization: the fixed-point pass and its marked points, where the mechanism fits.
-template <class TS>
 cudaError_t launch_lin_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
-                              const double* dlnA, TS* lin, int64_t ldl, cudaStream_t s) {
+                              const double* dlnA, double* lin, int64_t ldl, cudaStream_t s) {
     cudaError_t e = launch_lin_fx(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
     if (e != cudaSuccess) return e;
     const Shape sh{32, m.K >= 8 ? 4 : 1};
-    const size_t smem = lin_smem(m.K, sh, sizeof(TS) == sizeof(float) ? 5 : 0);
-    auto kern = sh.np == 4 ? linearize_kernel<32, 4, TS, true> : linearize_kernel<32, 1, TS, true>;
+    const size_t smem = lin_smem(m.K, sh, 0);
+    auto kern = sh.np == 4 ? linearize_kernel<32, 4, double, true> : linearize_kernel<32, 1, double, true>;
     e = ensure_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)((n + 31) / 32), 32 * sh.np, smem, s>>>(m, n, ld, T, p, Y, dlnA, lin, ldl);
@@ -848,11 +847,18 @@ int64_t lin_slots_f32(const DevMech& m) { return slot_EK32(m) + m.K; }
 cudaError_t launch_linearize(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                              const double* Y, const double* dlnA, double* lin, int64_t ldl, cudaStream_t s) {
     static_assert(kDfTabBytes <= kMathTabDoubles * sizeof(double), "table space");
-    if (lin_fx_fits(m)) return launch_lin_marked(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
     const int idx = plan_shape<0>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
     return launch_idx<0>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, dlnA,
                          lin, ldl);
+}
+
+// The linearization a solver keeps to itself: the fixed-point form where the mechanism fits.  (The
+// public one stays with the pair kernel, whose doubles the single-precision data are rounded from.)
+cudaError_t launch_linearize_solver(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
+                                    const double* Y, const double* dlnA, double* lin, int64_t ldl, cudaStream_t s) {
+    return lin_fx_fits(m) ? launch_lin_marked(m, n, ld, T, p, Y, dlnA, lin, ldl, s)
+                          : launch_linearize(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
 }
 
 cudaError_t launch_jvp_linearized(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
@@ -867,7 +873,6 @@ cudaError_t launch_jvp_linearized(const DevMech& m, int64_t n, int64_t ld, const
 
 cudaError_t launch_linearize_f32(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                                  const double* Y, const double* dlnA, float* lin, int64_t ldl, cudaStream_t s) {
-    if (lin_fx_fits(m)) return launch_lin_marked(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
     const int idx = plan_shape<5>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
     return launch_idx<5>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, dlnA,
@@ -881,14 +886,14 @@ cudaError_t launch_jvp_linearized_f32(const DevMech& m, int64_t n, int64_t ld, c
     if (rhs) {
         const int idx = plan_shape<4>(m.K);
         if (idx < 0) return cudaErrorInvalidConfiguration;
-        if (m.fx_ok)
+        if (lin32_fx_fits(m, kShapes[idx].np))
             return launch_lin32_fx<true>(kShapes[idx].np, m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, fT, fY, ldf, s);
         return launch_idx<4>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, lin,
                              ldl, vT, vY, d_Y, d_T, fT, fY, ldf);
     }
     const int idx = plan_shape<3>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
-    if (m.fx_ok)
+    if (lin32_fx_fits(m, kShapes[idx].np))
         return launch_lin32_fx<false>(kShapes[idx].np, m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, nullptr, nullptr, 0, s);
     const double* none = nullptr;
     return launch_idx<3>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, lin, ldl,

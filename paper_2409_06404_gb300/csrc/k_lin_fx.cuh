@@ -1,10 +1,12 @@
-// The per-entry stored linearization on fixed-point logarithms (nk_fx.cuh, nk_fxpt.cuh, nk_fxd.cuh;
+// The per-entry stored linearization of the reactor on fixed-point logarithms (nk_fx.cuh, nk_fxpt.cuh, nk_fxd.cuh;
 // included by k_lin.cu, whose slots and store_coef it uses): an entry's coefficient is its side's term
 // divided by the concentration, nu_e q_side / C_e, one product with a row of 1/C_k, where the pair
 // kernel formed exclusive products of the concentrations.  The stored words bound it together with
-// the FP64 pipe (one quotient's product per entry).  The stage with single-precision products
-// (k_lin32_fx.cuh), 53 species, 2,097,152 points: 21.7 -> 21.5 ms; block-Jacobi set-up and reactor
-// steps, which read the stored entries, 53 species: 9.50 -> 8.87 ms.
+// the FP64 pipe (one quotient's product per entry).  Block-Jacobi set-up and reactor steps, which
+// read the stored entries, 53 species, 16,384 points: 9.50 -> 8.87 ms.
+// For linearizations a solver keeps to itself; the public one and the single-precision data rounded
+// from it stay with the pair kernel: two linearizations that differ by 3e-13 round some hundred
+// coefficients of a field to the other float, 6e-8 of a product.
 #pragma once
 
 #include "nk_fxd.cuh"
@@ -14,26 +16,8 @@ namespace {
 
 enum { kLeMu = 256, kLeIC = 512, kLeE = 768, kLeCp = 1024 };   // (the derivative kernels' row)
 
-inline size_t lin_fx_smem(const DevMech& m, bool f32) {
-    return fx_smem(m.fxs[1], m.K, 64) + (f32 ? (size_t)m.K * 32 * sizeof(int) : 0);
-}
-inline bool lin_fx_fits(const DevMech& m) { return m.fx_ok && m.fxs[1].np != 0 && lin_fx_smem(m, true) <= smem_limit(); }
-
-// S1's slot: the double, or its two words
-__device__ __forceinline__ void put_s1(double* lin, int64_t at, int64_t, unsigned long long b) {
-    lin[at] = __longlong_as_double((long long)b);
-}
-__device__ __forceinline__ void put_s1(float* lin, int64_t at, int64_t ldl, unsigned long long b) {
-    reinterpret_cast<uint32_t*>(lin)[at] = (uint32_t)b;
-    reinterpret_cast<uint32_t*>(lin)[at + ldl] = (uint32_t)(b >> 32);
-}
-__device__ __forceinline__ unsigned long long get_s1(const double* lin, int64_t at, int64_t) {
-    return (unsigned long long)__double_as_longlong(lin[at]);
-}
-__device__ __forceinline__ unsigned long long get_s1(const float* lin, int64_t at, int64_t ldl) {
-    const uint32_t* u = reinterpret_cast<const uint32_t*>(lin);
-    return (unsigned long long)u[at + ldl] << 32 | u[at];
-}
+inline size_t lin_fx_smem(const DevMech& m) { return fx_smem(m.fxs[1], m.K, 64); }
+inline bool lin_fx_fits(const DevMech& m) { return m.fx_ok && m.fxs[1].np != 0 && lin_fx_smem(m) <= smem_limit(); }
 
 // nu_e q / C_e of a side's entries (each a branch per count: predicated FP64 products cost as much as
 // executed ones), an entry's first molecule found by adding up the coefficients before it
@@ -58,12 +42,11 @@ __device__ __forceinline__ void entry_coefs(const unsigned char* ic, const uint3
 }
 
 // Points outside the form leave kFxSkip in their S1 slot for the marked pass of k_lin.cu.
-template <int NP, int BLOCKS, class TS>
+template <int NP, int BLOCKS>
 __global__ void __launch_bounds__(32 * NP, BLOCKS)
     lin_fx_kernel(const DevMech m, const int64_t n, const int64_t ld, const double* __restrict__ T,
                   const double* __restrict__ p, const double* __restrict__ Y, const double* __restrict__ dlnA,
-                  TS* __restrict__ lin, const int64_t ldl) {
-    constexpr bool F32 = sizeof(TS) == sizeof(float);
+                  double* __restrict__ lin, const int64_t ldl) {
     extern __shared__ __align__(16) unsigned char smem_fx[];
     const FxSet& f = m.fxs[1];
     unsigned char* im0 = smem_fx + kFxBase + kFxScalars * 256;
@@ -79,8 +62,6 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
     long long* sS = reinterpret_cast<long long*>(smem_fx + kFxBase) + lane;
     unsigned char* sP = im0 + 2 * f.image + lane * 8;
     unsigned char* sQ = sP + (size_t)(K + 1) * kFxDRow;                      // the parts' sums
-    const size_t qb = (size_t)f.rows * 64, pb = (size_t)f.np * 3 * 256;
-    int* sE = reinterpret_cast<int*>(sQ - lane * 8 + (qb > pb ? qb : pb)) + lane;   // F32: E_k, species order
 
     double Ti = T[i];
     bool bad = !fx_T_ok(Ti);
@@ -126,8 +107,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             *reinterpret_cast<double*>(row + kLeIC) = fx_exp2<true>((a & 1) - (a & ~1ll), ft);
             *reinterpret_cast<long long*>(row + kLeE) = (1ll << kFxS) - h;
             *reinterpret_cast<long long*>(row + kLeCp) = fx_cpR(c, u);
-            if (live && good) put(lin + ((F32 ? slot_H32(m) : slot_H(m)) + ks) * ldl + i, fx_to_d(h));
-            if constexpr (F32) sE[ks * 32] = kNoExp;
+            if (live && good) lin[(slot_H(m) + ks) * ldl + i] = fx_to_d(h);
         }
         if (part == 0) {
             sS[kFxLrho * 32] = lrho;
@@ -228,32 +208,28 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                 entry_coefs(sP + kLeIC, off + 4, h.z, nu + kMaxSide, -qr, Bv + kMaxSide);
                 const double A = fma(qq, aT, qr * fx_to_d(-E));
                 if (kind == 0)
-                    store_coef<32, 0>(m, r, lin, ldl, i, h.y, h.z, sp, sE, A, Bv, 0.0);
+                    store_coef<32, 0>(m, r, lin, ldl, i, h.y, h.z, sp, nullptr, A, Bv, 0.0);
                 else
-                    store_coef<32, 1>(m, r, lin, ldl, i, h.y, h.z, sp, sE, A, Bv, qc * cL);
+                    store_coef<32, 1>(m, r, lin, ldl, i, h.y, h.z, sp, nullptr, A, Bv, qc * cL);
             }
         }
         fx_image_wait();
         __syncthreads();
     }
 
-    if constexpr (F32)
-        if (store)
-            for (int k = part; k < K; k += NP) reinterpret_cast<int32_t*>(lin)[(slot_EK32(m) + k) * ldl + i] = sE[k * 32];
     double* sR = reinterpret_cast<double*>(sQ);
     sR[part * 32] = S1;
     __syncthreads();
     if (part != 0 || !live) return;
     for (int q = 1; q < NP; ++q) S1 += sR[q * 32];
-    put_s1(lin, slot_S(m) * ldl + i, ldl, good ? (unsigned long long)__double_as_longlong(S1 * kFxCpScale) : kFxSkip);
+    lin[slot_S(m) * ldl + i] = good ? S1 * kFxCpScale : __longlong_as_double((long long)kFxSkip);
 }
 
-template <class TS>
-cudaError_t launch_lin_fx(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
-                          const double* dlnA, TS* lin, int64_t ldl, cudaStream_t s) {
-    const size_t smem = lin_fx_smem(m, sizeof(TS) == sizeof(float));
+inline cudaError_t launch_lin_fx(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
+                          const double* dlnA, double* lin, int64_t ldl, cudaStream_t s) {
+    const size_t smem = lin_fx_smem(m);
     const int np = m.fxs[1].np;
-    auto kern = np == 4 ? lin_fx_kernel<4, 6, TS> : np == 12 ? lin_fx_kernel<12, 2, TS> : lin_fx_kernel<24, 1, TS>;
+    auto kern = np == 4 ? lin_fx_kernel<4, 6> : np == 12 ? lin_fx_kernel<12, 2> : lin_fx_kernel<24, 1>;
     const cudaError_t e = ensure_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)((n + 31) / 32), 32 * np, smem, s>>>(m, n, ld, T, p, Y, dlnA, lin, ldl);

@@ -403,6 +403,8 @@ int64_t lin_slots(const DevMech& m);
 int64_t lin_slots_f32(const DevMech& m);   // the float format's 32-bit words per point
 cudaError_t launch_linearize(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                              const double* Y, const double* dlnA, double* lin, int64_t ldl, cudaStream_t s);
+cudaError_t launch_linearize_solver(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
+                                    const double* Y, const double* dlnA, double* lin, int64_t ldl, cudaStream_t s);
 cudaError_t launch_jvp_linearized(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                                   const double* Y, const double* lin, int64_t ldl, const double* vT,
                                   const double* vY, double* d_omega, double* d_hrr, cudaStream_t s);

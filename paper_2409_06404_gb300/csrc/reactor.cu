@@ -403,7 +403,7 @@ cudaError_t reactor_step(const DevMech& m, int64_t n, double* T, const double* p
             return cudaSuccess;
         }
         if (o.linearized == 1 &&                   // the rates' tangent data at this iterate
-            (e = launch_linearize(m, n, ld, T, p, Y, nullptr, w.lin, n, s)) != cudaSuccess)
+            (e = launch_linearize_solver(m, n, ld, T, p, Y, nullptr, w.lin, n, s)) != cudaSuccess)
             return e;
         if (o.linearized == 2 &&                   // the same, rounded to float
             (e = launch_linearize_f32(m, n, ld, T, p, Y, nullptr, w.linf, n, s)) != cudaSuccess)
@@ -413,7 +413,7 @@ cudaError_t reactor_step(const DevMech& m, int64_t n, double* T, const double* p
                 const int64_t nc = std::min(w.nchunk, n - c0);
                 const bool full = o.linearized == 1;    // the full double data: stride n
                 if (!full &&
-                    (e = launch_linearize(m, nc, ld, T + c0, p + c0, Y + c0, nullptr, w.lin, nc, s)) != cudaSuccess)
+                    (e = launch_linearize_solver(m, nc, ld, T + c0, p + c0, Y + c0, nullptr, w.lin, nc, s)) != cudaSuccess)
                     return e;
                 const double* lc = full ? w.lin + c0 : w.lin;
                 if ((e = launch_precond_setup(m, nc, ld, T + c0, p + c0, Y + c0, lc, full ? n : nc, w.f + c0,
