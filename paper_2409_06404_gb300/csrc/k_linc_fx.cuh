@@ -8,7 +8,7 @@
 // derivatives are products in doubles).  FP64 helpers of the rare cases (nu other than 1, falloff)
 // stay out of line: as predicated instructions they cost the pipe as much as executed ones.
 // One linearization with its sources and the products of a linearly implicit stage, 53 species,
-// 2,097,152 points: 37.2 -> 30.8 ms for the stage; error against 64-bit sums 2.8e-13 -> 4e-14.
+// 262,144 points: 37.3 -> 30.1 ms for the stage; error against 64-bit sums 3e-13 -> 4e-14.
 #pragma once
 
 #include "nk_fxd.cuh"
@@ -299,12 +299,45 @@ static __device__ __noinline__ double side_edge(const RxnRec* rec, const double*
 // r_k in a row per species (slot order), the reactions' dq staged per chunk and summed by species:
 // 34 KB of shared memory at 53 species, 24 warps per SM, where a row of d omega_k partials per warp
 // held it at 12, and every point sum is made once instead of once per warp.
+// dC_k has a row too: the efficiency sums are one operation and no global load of the state per entry.
 constexpr int kPcScalars = 4;                       // dT/T, d rho/rho, rho, d(p/RT)
 
 inline size_t jvpc_fx_smem(const DevMech& m) {
     const FxSet& f = m.fxs[2];
     const size_t q = (size_t)f.rows * 256, part = (size_t)f.np * 3 * 256;
-    return kPcScalars * 256 + 2 * (size_t)f.image + (size_t)f.row * (m.K + 1) + (q > part ? q : part);
+    return kPcScalars * 256 + 2 * (size_t)f.image + (size_t)f.row * (m.K + 1) + (size_t)m.K * 256 + (q > part ? q : part);
+}
+
+// the stored words of one reaction
+struct WordsC {
+    double A, Vf, Vb, L;
+    int nu;
+};
+__device__ __forceinline__ void load_words(const DevMech& m, const unsigned char* im, int q, const double* o, int64_t ldl,
+                                           WordsC& w) {
+    const long long hd = reinterpret_cast<const longlong2*>(im + q * (int)sizeof(FxRxn))[1].y;
+    const int r = (int)(hd >> 48);
+    w.A = __ldcs(o + (int64_t)r * ldl);
+    w.Vf = __ldcs(o + (cs_Vf(m) + r) * ldl);
+    w.Vb = __ldcs(o + (cs_Vb(m) + r) * ldl);
+    w.L = ((int)hd >> 8 & 3) != 0 ? __ldcs(o + (cs_L(m) + (r - m.R_el)) * ldl) : 0.0;
+    w.nu = __ldg(m.fx_nu1 + r);
+}
+
+// The stored words of a chunk's reactions into L2, while the chunk before is gathered: a row of the
+// block's 32 points is 256 bytes, two lines.  (Words loaded a reaction ahead into registers spilled
+// 240 bytes at the kernel's 80 registers.)
+__device__ __forceinline__ void prefetch_words(const DevMech& m, const FxSet& f, int np, const unsigned char* im,
+                                               const double* lin, int64_t ldl, int64_t n) {
+    const int total = im[f.image_parts + np] * 8;
+    for (int t = threadIdx.x; t < total; t += blockDim.x) {
+        const long long hd = reinterpret_cast<const longlong2*>(im + (t >> 3) * (int)sizeof(FxRxn))[1].y;
+        const int r = (int)(hd >> 48), word = t >> 1 & 3;
+        if (word == 3 && ((int)hd >> 8 & 3) == 0) continue;
+        const int64_t row = word == 0 ? r : word == 1 ? cs_Vf(m) + r : word == 2 ? cs_Vb(m) + r : cs_L(m) + (r - m.R_el);
+        const int64_t pt = min((int64_t)blockIdx.x * 32 + (t & 1) * 16, n - 1);
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(lin + row * ldl + pt));
+    }
 }
 
 template <int NP, bool RHS>
@@ -325,7 +358,8 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 6 : NP == 8 ? 3 : NP == 16 
     const int64_t i = live ? i0 : n - 1;
     double* sV = reinterpret_cast<double*>(smem_fx) + lane;
     unsigned char* sP = im0 + 2 * f.image + lane * 8;
-    unsigned char* sQ = sP + (size_t)(K + 1) * 256;
+    double* sC = reinterpret_cast<double*>(sP + (size_t)(K + 1) * 256);          // dC_k, species order
+    unsigned char* sQ = sP + (size_t)(2 * K + 1) * 256;
     double* sR = reinterpret_cast<double*>(sQ);
     {
         double s = 0.0, ds = 0.0;
@@ -356,7 +390,9 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 6 : NP == 8 ? 3 : NP == 16 
 #pragma unroll 1
     for (int k = part; k < K; k += NP) {
         const int ks = __ldg(&f.sp[k].k);
-        *reinterpret_cast<double*>(sP + k * 256) = fma(vY[(int64_t)ks * ld + i], lin[(cs_iY(m) + ks) * ldl + i], sV[32]);
+        const double v = vY[(int64_t)ks * ld + i], ar = sV[32];
+        *reinterpret_cast<double*>(sP + k * 256) = fma(v, lin[(cs_iY(m) + ks) * ldl + i], ar);
+        sC[ks * 32] = fma(sV[64] * __ldg(m.invW + ks), v, ar * lin[(cs_C(m) + ks) * ldl + i]);
     }
     fx_image_wait();
     __syncthreads();
@@ -364,6 +400,7 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 6 : NP == 8 ? 3 : NP == 16 
     double w[kFxOwn];
 #pragma unroll
     for (int j = 0; j < kFxOwn; ++j) w[j] = 0.0;
+    const double* o = lin + i;
     for (int c = 0; c < f.nchunk; ++c) {
         const unsigned char* im = im0 + (c & 1) * f.image;
         fx_image_load(f, c + 1, im0 + ((c + 1) & 1) * f.image);
@@ -373,45 +410,38 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 6 : NP == 8 ? 3 : NP == 16 
             const longlong2* rec = reinterpret_cast<const longlong2*>(im + q * (int)sizeof(FxRxn));
             const long long hd = rec[1].y;
             const int info = (int)hd, r = (int)(hd >> 48), kind = info >> 8 & 3;
-            const double* o = lin + i;
-            const double A = __ldcs(o + (int64_t)r * ldl), Vf = __ldcs(o + (cs_Vf(m) + r) * ldl),
-                         Vb = __ldcs(o + (cs_Vb(m) + r) * ldl);
-            const double Lc = kind != 0 ? __ldcs(o + (cs_L(m) + (r - m.R_el)) * ldl) : 0.0;
+            WordsC v;
+            load_words(m, im, q, o, ldl, v);
             const uint4 re = reinterpret_cast<const uint4*>(rec)[2], pr = reinterpret_cast<const uint4*>(rec)[3];
             const int nr = info & 15, np = info >> 4 & 15;
             double gf = side_flat(sP, re, nr), gb = side_flat(sP, pr, np);
-            const int nu = __ldg(m.fx_nu1 + r);        // the stored V carry the first entries' coefficients
+            const int nu = v.nu;                       // the stored V carry the first entries' coefficients
             if ((nu & 15) != 1) gf = over_nu(gf, nu & 15);
             if ((nu >> 4) != 1) gb = over_nu(gb, nu >> 4);
             double dq;
             if (!nonfinite(gf) && !nonfinite(gb)) {
-                dq = fma(Vf, gf, fma(Vb, gb, A * sV[0]));
+                dq = fma(v.Vf, gf, fma(v.Vb, gb, v.A * sV[0]));
             } else {
-                dq = side_edge(m.rxn + r, m.invW, Vf, gf, Vb, gb, A * sV[0], lin + cs_iY(m) * ldl + i,
+                dq = side_edge(m.rxn + r, m.invW, v.Vf, gf, v.Vb, gb, v.A * sV[0], lin + cs_iY(m) * ldl + i,
                                ExactCtx{lin + cs_C(m) * ldl + i, vY + i, ldl, ld, sV[64], sV[32]});
             }
             if (kind != 0) {
-                const int4 x = __ldg(reinterpret_cast<const int4*>(m.fx_extra + (info >> 16)));
-                // d[M] = d(p/RT) + sum (eps - 1) dC, dC_k = C_k d rho/rho + rho dY_k/W_k
-                double sc = 0.0, sy = 0.0;
+                const int2 e = __ldg(reinterpret_cast<const int2*>(m.fx_extra + (info >> 16)));
+                double dM = sV[96];                    // d[M] = d(p/RT) + sum (eps - 1) dC
 #pragma unroll 1
-                for (int j = x.x; j < x.y; ++j) {
-                    const FxEff* t = m.fx_eff + j;
-                    const int k = __ldg(&t->sp);
-                    sc = fma(__ldg(m.eff_m1 + j), lin[(cs_C(m) + k) * ldl + i], sc);
-                    sy = fma(__ldg(&t->wd), vY[(int64_t)k * ld + i], sy);
-                }
-                dq = fma(Lc, fma(sV[32], sc, fma(sV[64] * m.fx_maxw, sy, sV[96])), dq);
+                for (int j = e.x; j < e.y; ++j) dM = fma(__ldg(m.eff_m1 + j), sC[__ldg(&m.fx_eff[j].sp) * 32], dM);
+                dq = fma(v.L, dM, dq);
             }
             *reinterpret_cast<double*>(sQ + q * 256) = dq;
         }
+        fx_image_wait();
         __syncthreads();
+        if (c + 1 < f.nchunk) prefetch_words(m, f, NP, im0 + ((c + 1) & 1) * f.image, lin, ldl, n);
         const uint32_t* spec = reinterpret_cast<const uint32_t*>(im + f.image_spec);
         const unsigned char* list = im + f.image_list;
 #pragma unroll
         for (int j = 0; j < kFxOwn; ++j)
             if (part + NP * j < K) w[j] = fx_gather(spec[part + NP * j], list, sQ, w[j]);
-        fx_image_wait();
         __syncthreads();
     }
     // d omega_k in species order (r_k is dead), then the shared epilogue
