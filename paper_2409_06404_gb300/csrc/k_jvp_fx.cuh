@@ -5,7 +5,7 @@
 // dY_k/Y_k (a float pair), e_k = 1 - h_k/RT = T d mu_k/dT (natural units) and c_p,k/R, the last two
 // as integers: a reaction's temperature derivatives are integer sums over its molecules where the
 // pair kernel (k_jvp.cuh) evaluated three reaction polynomials.  With theta = dT/T,
-// s = T d ln k/dT (53 species / 325 reactions, 512,000 points: 10.9 -> 7.4 ms; error against 64-bit
+// s = T d ln k/dT (53 species / 325 reactions, 512,000 points: 10.9 -> 7.1 ms; error against 64-bit
 // sums 3e-13 -> 4e-14):
 //   dq = q_f (theta s + sum_reactants r) - q_r (theta (s + sum nu e) + sum_products r).
 #pragma once

@@ -9,7 +9,7 @@
 // terms and one addition per molecule), and issue slots and the FP64 pipe bound it about equally
 // (61% and 56% busy).  Accumulators in registers, loops over species not unrolled and the falloff
 // out of line: the unrolled form of the same kernel measured 18 ms, waiting for instructions.
-// 53 species, 2,097,152 points: 22.0 -> 13.6 ms; its error against 64-bit sums fell from 3e-13 to
+// 53 species, 2,097,152 points: 22.0 -> 13.9 ms; its error against 64-bit sums fell from 3e-13 to
 // 3e-14 (2-norm).
 #pragma once
 
@@ -51,7 +51,7 @@ static __device__ __noinline__ float fx_troe_float(const TroeRecF* t, float Mf, 
 // MIXED (NK_MIXED): ln k_f and the whole falloff in single precision, operation by operation as the
 // pair kernel's mixed form has them (so its results stay, to some 1e-13); concentrations, K_c, the
 // difference and the sums as in the FP64 form.  Rates and transport at 120 species / 700
-// reactions, 110,592 points: 7.06 -> 5.41 ms (all of it the rates').
+// reactions, 110,592 points: 7.05 -> 5.21 ms (all of it the rates').
 template <int NP, bool RHS, bool MIXED>
 __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
     rates_fx_kernel(const DevMech m, const int64_t n, const int64_t ld, const double* __restrict__ T,

@@ -7,8 +7,8 @@
 // molecules B_r + Y_k sum over its efficiencies w X_r, X_r = (F_r + B_r) px/([M]/rho') (px = 1 for
 // third-body reactions), and the ln A gradient of a reaction is the sum of F + B over the block's
 // points, each lane summing one reaction's row.  A persistent grid walks the tiles of 32 points.
-// Rates and their gradients through autograd, 53 species / 325 reactions, 200,003 points: 9.2 -> 6.1
-// ms (of which the rates 2.1 -> 1.3); error against 64-bit sums 6e-13 -> 4e-14.
+// Rates and their gradients through autograd, 53 species / 325 reactions, 200,003 points: 8.8 -> 5.3
+// ms (of which the rates 2.1 -> 1.3); error against 64-bit sums 3e-13 -> 6e-14.
 #pragma once
 
 #include "nk_fxd.cuh"
