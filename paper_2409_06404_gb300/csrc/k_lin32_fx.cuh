@@ -5,9 +5,9 @@
 // points).  A species' terms are summed in the order of those rounds (FxTerm32) and the point sums
 // by the same parts, so the results are the same bits.  Load latency bounds it (waits on stored words
 // 4.2 cycles per issue, issue slots 51% busy), so a reaction's words are loaded while the one before
-// is summed, and all parts load the state.  53 species, 65,536 points: 0.38 ms per product (1.7 TB/s
-// of the stored words); the single-precision stage of 175,616 points,
-// with its ten products: 21.9 -> 15.8 ms.
+// is summed, and all parts load the state.  53 species, 2,097,152 points: 12.6 -> 9.0 ms per product
+// (2.3 TB/s of the stored words); the single-precision stage of 175,616 points with its ten
+// products: 21.7 -> 15.8 ms.
 #pragma once
 
 #include "nk_fxpt.cuh"

@@ -8,7 +8,8 @@
 // derivatives are products in doubles).  FP64 helpers of the rare cases (nu other than 1, falloff)
 // stay out of line: as predicated instructions they cost the pipe as much as executed ones.
 // One linearization with its sources and the products of a linearly implicit stage, 53 species,
-// 262,144 points: 37.3 -> 30.1 ms for the stage; error against 64-bit sums 3e-13 -> 4e-14.
+// 262,144 points: 37.1 -> 30.1 ms for the stage (at 2,097,152 points the linearization 53.6 ->
+// 27.7 ms, a product 24.0 -> 20.9); error against 64-bit sums 3e-13 -> 4e-14.
 #pragma once
 
 #include "nk_fxd.cuh"
