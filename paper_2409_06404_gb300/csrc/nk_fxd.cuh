@@ -37,6 +37,12 @@ __device__ __forceinline__ dfl split_pair(double v) {
     const MantPair a = mant_pair(v);
     return df_ldexp(a.m, a.e);
 }
+// v 2^s as a pair, for a double of any size below 2^100: what a pair cannot carry (below 2^-126)
+// goes to zero
+__device__ __forceinline__ dfl split_pair_scaled(double v, int s) {
+    const MantPair a = mant_pair(v);
+    return a.e + s < -126 ? dfl{0.0f, 0.0f} : df_ldexp(a.m, a.e + s);
+}
 // |y| in [2^-100, 2^100)
 __device__ __forceinline__ bool log_range_ok(double y) {
     const unsigned e = (unsigned)((unsigned long long)__double_as_longlong(y) >> 52) & 0x7ffu;
@@ -47,7 +53,8 @@ __device__ __forceinline__ dfl fxc_ln2() { return {0.693147182464599609375f, -1.
 // As fx_third_body, and d ln[M]: with [M] = rho' z, z = s + sum (eps - 1) Y/W, s = sum Y/W, at
 // d rho/rho = arho and d(p/RT) = -theta p/RT it is
 //   (arho (z - s) - theta s + sum (eps - 1) dY/W) / z,
-// the sum in double (terms of any size), the rest in pairs of z's unit.
+// the sum in double (its terms are in the pairs' range, but where they cancel it may be of any size
+// below that), the rest in pairs of z's unit.
 __device__ __forceinline__ long long fx_third_body_d(const DevMech& m, int eff0, int eff1, const double* Y,
                                                      const double* vY, int64_t ld, int64_t i, long long sum, dfl theta,
                                                      dfl arho, const FxTab& t, long long& lM, dfl& dlnM) {
@@ -66,7 +73,7 @@ __device__ __forceinline__ long long fx_third_body_d(const DevMech& m, int eff0,
         }
     }
     lM = fx_log2_int((unsigned long long)(z > 0 ? z : z < 0 ? -z : 1ll), 60 - m.fx_eff_shift, t) + m.fx_lmaxw;
-    dfl d = df_ldexp(split_pair(dz), 12 - m.fx_eff_shift);
+    dfl d = split_pair_scaled(dz, 12 - m.fx_eff_shift);
     d = df_fma(arho, fx_to_pair(z - s), d);
     d = df_add(d, df_neg(df_mul(theta, fx_to_pair(s))));
     dlnM = df_div(z < 0 ? df_neg(d) : d, fx_to_pair(z < 0 ? -z : z != 0 ? z : 1ll));
