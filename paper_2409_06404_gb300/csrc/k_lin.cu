@@ -746,6 +746,8 @@ constexpr auto kernel_of() {
         return jvp_lin32_kernel<kShapes[S].blk, kShapes[S].np, true>;
     else if constexpr (MODE == 5)
         return linearize_kernel<kShapes[S].blk, kShapes[S].np, float>;
+    else if constexpr (MODE == 7)
+        return linearize_kernel<kShapes[S].blk, kShapes[S].np, double, true>;
     else
         return linearize_kernel<kShapes[S].blk, kShapes[S].np, double>;
 }
@@ -759,7 +761,7 @@ const void* kernel_ptr(int idx, std::integer_sequence<int, S...>) {
 // linearization: the pair tables and C_k; apply: dC_k and the d omega_k row (and the part sums
 // of the single-precision apply)
 size_t lin_smem(int K, const Shape& sh, int mode) {
-    if (mode == 0 || mode == 5)
+    if (mode == 0 || mode == 5 || mode == 7)
         return (size_t)kMathTabDoubles * sizeof(double) + (size_t)K * sh.blk * (mode == 5 ? 12 : 8);
     if (mode == 3 || mode == 4) return lin32_smem(K, sh.blk, sh.np);
     return (size_t)2 * K * sh.blk * sizeof(double);
@@ -830,13 +832,17 @@ cudaError_t launch_lin_marked(const DevMech& m, int64_t n, int64_t ld, const dou
                               const double* dlnA, double* lin, int64_t ldl, cudaStream_t s) {
     cudaError_t e = launch_lin_fx(m, n, ld, T, p, Y, dlnA, lin, ldl, s);
     if (e != cudaSuccess) return e;
-    const Shape sh{32, m.K >= 8 ? 4 : 1};
-    const size_t smem = lin_smem(m.K, sh, 0);
-    auto kern = sh.np == 4 ? linearize_kernel<32, 4, double, true> : linearize_kernel<32, 1, double, true>;
-    e = ensure_smem((const void*)kern, smem);
-    if (e != cudaSuccess) return e;
-    kern<<<(unsigned)((n + 31) / 32), 32 * sh.np, smem, s>>>(m, n, ld, T, p, Y, dlnA, lin, ldl);
-    return cudaGetLastError();
+    // Four parts while that takes no more than one wave of blocks (four per SM), the planned shape
+    // above: all points marked, 53 species, 16,384 points: 0.42 ms by four parts, 1.18 by the planned
+    // shape, 65,536 points: 1.75 and 1.60; 9 species, 262,144 points: 0.68 and 0.48.
+    int idx = plan_shape<0>(m.K);
+    if (idx < 0) return cudaErrorInvalidConfiguration;
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    if (m.K >= 8 && (n + 31) / 32 <= 4 * sms) idx = kNumShapes - 1;
+    static_assert(kShapes[kNumShapes - 1].blk == 32 && kShapes[kNumShapes - 1].np == 4, "four parts");
+    return launch_idx<7>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, dlnA, lin, ldl);
 }
 
 }  // namespace

@@ -41,8 +41,9 @@ __device__ __forceinline__ void entry_coefs(const unsigned char* ic, const uint3
     }
 }
 
-// Points outside the form leave kFxSkip in their S1 slot for the marked pass of k_lin.cu.
-template <int NP, int BLOCKS>
+// Blocks with a point outside the form (as in k_linc_fx.cuh) leave kFxSkip in their points' S1 slot for
+// the marked pass of k_lin.cu.
+template <int NP, int OWN, int BLOCKS>
 __global__ void __launch_bounds__(32 * NP, BLOCKS)
     lin_fx_kernel(const DevMech m, const int64_t n, const int64_t ld, const double* __restrict__ T,
                   const double* __restrict__ p, const double* __restrict__ Y, const double* __restrict__ dlnA,
@@ -50,10 +51,6 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
     extern __shared__ __align__(16) unsigned char smem_fx[];
     const FxSet& f = m.fxs[1];
     unsigned char* im0 = smem_fx + kFxBase + kFxScalars * 256;
-    fx_image_load(f, 0, im0);
-    const FxTab ft = stage_fx_tables(reinterpret_cast<uint32_t*>(smem_fx), m.fx_tab);
-    const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem_fx + kFxTabBytes), m);
-    __syncthreads();
     const int K = m.K;
     const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
     const int64_t i0 = (int64_t)blockIdx.x * 32 + lane;
@@ -63,36 +60,52 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
     unsigned char* sP = im0 + 2 * f.image + lane * 8;
     unsigned char* sQ = sP + (size_t)(K + 1) * kFxDRow;                      // the parts' sums
 
-    double Ti = T[i];
-    bool bad = !fx_T_ok(Ti);
-    if (bad) Ti = 1000.0;
+    // a block with a point outside the form leaves here, all its points marked (as in k_jvp_fx.cuh; one
+    // zero mass fraction in every block, 53 species, 262,144 points: 9.1 -> 6.1 ms)
+    const double Ti = T[i], pi = p[i];
     const unsigned long long Tb = (unsigned long long)__double_as_longlong(Ti);
+    double y[OWN];                                           // (all loads in flight at once)
+#pragma unroll
+    for (int j = 0; j < OWN; ++j) y[j] = part + NP * j < K ? Y[(int64_t)__ldg(&f.sp[part + NP * j].k) * ld + i] : 1.0;
+    fx_image_load(f, 0, im0);
+    const FxTab ft = stage_fx_tables(reinterpret_cast<uint32_t*>(smem_fx), m.fx_tab);
+    const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem_fx + kFxTabBytes), m);
+    bool bad = !fx_T_ok(Ti) || !fx_p_ok(pi);
+#pragma unroll
+    for (int j = 0; j < OWN; ++j) bad |= !fx_y_ok(y[j]);
+    if (__syncthreads_or(bad) != 0) {
+        if (part == 0 && live) lin[slot_S(m) * ldl + i] = __longlong_as_double((long long)kFxSkip);
+        fx_image_wait();
+        return;
+    }
     {
         unsigned long long z = 0, zc = 0;
-#pragma unroll 1
-        for (int k = part; k < K; k += NP) {
-            const FxSpecies* sp = f.sp + k;
-            const double y = Y[(int64_t)__ldg(&sp->k) * ld + i];
-            fx_add_fraction((unsigned long long)__double_as_longlong(y), __ldg((const long long*)&sp->w), z, zc, bad);
-            bad |= !log_range_ok(y);
+#pragma unroll
+        for (int j = 0; j < OWN; ++j) {
+            if (part + NP * j >= K) break;
+            fx_add_fraction((unsigned long long)__double_as_longlong(y[j]), __ldg((const long long*)&f.sp[part + NP * j].w), z, zc, bad);
         }
-        if (part == 0) bad |= !fx_point_scalars(m, Tb, p[i], sS, ft);
         reinterpret_cast<unsigned long long*>(sQ)[(2 * part) * 32] = z;
-        reinterpret_cast<unsigned long long*>(sQ)[(2 * part + 1) * 32] = bad ? kFxPoison : zc;
+        reinterpret_cast<unsigned long long*>(sQ)[(2 * part + 1) * 32] = zc;
     }
+    if (part == 0) fx_point_scalars(m, Tb, pi, sS, ft);
     __syncthreads();
     FxT P;
     P.lt = fx_frac63((unsigned long long)sS[kFxLT * 32] << 11);
     P.v = fx_frac63((unsigned long long)sS[kFxV * 32]);
-    bool good;
     {
         unsigned long long z = 0, zc = 0;
         for (int q = 0; q < NP; ++q) {
             z += reinterpret_cast<unsigned long long*>(sQ)[(2 * q) * 32];
             zc += reinterpret_cast<unsigned long long*>(sQ)[(2 * q + 1) * 32];
         }
-        good = !fx_sums_bad(z, zc);
-        const long long lrho = good ? sS[kFxLpRT * 32] - fx_log2_int(z, 60, ft) - m.fx_lmaxw : 0;
+        // (the conditions on the point sums)
+        if (__any_sync(0xffffffffu, fx_sums_bad(z, zc))) {
+            if (part == 0 && live) lin[slot_S(m) * ldl + i] = __longlong_as_double((long long)kFxSkip);
+            fx_image_wait();
+            return;
+        }
+        const long long lrho = sS[kFxLpRT * 32] - fx_log2_int(z, 60, ft) - m.fx_lmaxw;
         const FxFrac u = fx_frac_T(Tb);
 #pragma unroll 1
         for (int k = part; k < K; k += NP) {
@@ -100,21 +113,20 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             const int ks = __ldg(&sp->k);
             unsigned char* row = sP + k * kFxDRow;
             const int64_t* c = fx_range(sp, Ti);
-            const long long a = good ? fx_log2_conc((unsigned long long)__double_as_longlong(Y[(int64_t)ks * ld + i]), __ldg((const long long*)&sp->lw) + lrho, ft) : 0;
+            const long long a = fx_log2_conc((unsigned long long)__double_as_longlong(Y[(int64_t)ks * ld + i]), __ldg((const long long*)&sp->lw) + lrho, ft);
             const long long h = fx_hRT(c, P, u);
             *reinterpret_cast<long long*>(row) = a;
             *reinterpret_cast<long long*>(row + kLeMu) = a + (fx_mu0(c, P, u) & ~1ll);
             *reinterpret_cast<double*>(row + kLeIC) = fx_exp2<true>((a & 1) - (a & ~1ll), ft);
             *reinterpret_cast<long long*>(row + kLeE) = (1ll << kFxS) - h;
             *reinterpret_cast<long long*>(row + kLeCp) = fx_cpR(c, u);
-            if (live && good) lin[(slot_H(m) + ks) * ldl + i] = fx_to_d(h);
+            if (live) lin[(slot_H(m) + ks) * ldl + i] = fx_to_d(h);
         }
         if (part == 0) {
             sS[kFxLrho * 32] = lrho;
-            sS[kFxSum * 32] = good ? (long long)z : 0;
+            sS[kFxSum * 32] = (long long)z;
         }
     }
-    const bool store = live && good;
     fx_image_wait();
     __syncthreads();
 
@@ -198,7 +210,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             const double qc = qq;
             if (kind == 1 && zero) qq = qf = qr = 0.0;
             S1 = fma(qq, fx_to_d(Cp), S1);
-            if (store) {
+            if (live) {
                 const int4* xr = reinterpret_cast<const int4*>(m.rxn + r) + 6;
                 const int4 h = __ldg(xr), s0 = __ldg(xr + 2), s1 = __ldg(xr + 3), u0 = __ldg(xr + 4), u1 = __ldg(xr + 5);
                 const int sp[2 * kMaxSide] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
@@ -222,14 +234,14 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
     __syncthreads();
     if (part != 0 || !live) return;
     for (int q = 1; q < NP; ++q) S1 += sR[q * 32];
-    lin[slot_S(m) * ldl + i] = good ? S1 * kFxCpScale : __longlong_as_double((long long)kFxSkip);
+    lin[slot_S(m) * ldl + i] = S1 * kFxCpScale;
 }
 
 inline cudaError_t launch_lin_fx(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
                           const double* dlnA, double* lin, int64_t ldl, cudaStream_t s) {
     const size_t smem = lin_fx_smem(m);
     const int np = m.fxs[1].np;
-    auto kern = np == 4 ? lin_fx_kernel<4, 6> : np == 12 ? lin_fx_kernel<12, 2> : lin_fx_kernel<24, 1>;
+    auto kern = np == 4 ? lin_fx_kernel<4, 8, 6> : np == 12 ? lin_fx_kernel<12, 6, 2> : lin_fx_kernel<24, 6, 1>;
     const cudaError_t e = ensure_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)((n + 31) / 32), 32 * np, smem, s>>>(m, n, ld, T, p, Y, dlnA, lin, ldl);

@@ -529,14 +529,16 @@ cudaError_t launch_idx(int idx, std::integer_sequence<int, S...>, int K, int64_t
     return e;
 }
 
-// The marked points of the fixed-point pass.
+// The marked points of the fixed-point pass, by the planned shape's parts (9 species, 262,144 points, all
+// of them marked: 0.67 ms by four parts, 0.54 by the planned one).
 template <bool OUT>
 cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
                           const double* dlnA, double* lin, int64_t ldl, double* omega, double* hrr, cudaStream_t s) {
-    int np = m.K >= 8 ? 4 : 1;
-    while (np > 1 && linc_smem(m.K, 32, np, OUT) > smem_limit()) np = 1;
+    const int idx = plan_shape<OUT ? 1 : 0>(m.K);
+    if (idx < 0) return cudaErrorInvalidConfiguration;
+    const int np = kShapes[idx].np;
     const size_t smem = linc_smem(m.K, 32, np, OUT);
-    auto kern = np == 4 ? linc_kernel<32, 4, OUT, true> : linc_kernel<32, 1, OUT, true>;
+    auto kern = np == 4 ? linc_kernel<32, 4, OUT, true> : np == 2 ? linc_kernel<32, 2, OUT, true> : linc_kernel<32, 1, OUT, true>;
     const cudaError_t e = ensure_smem((const void*)kern, smem);
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)((n + 31) / 32), 32 * np, smem, s>>>(m, n, ld, T, p, Y, dlnA, lin, ldl, omega, hrr);

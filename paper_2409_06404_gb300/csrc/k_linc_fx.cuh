@@ -23,13 +23,14 @@ enum { kLcMu = 256, kLcE = 768, kLcCp = 1024 };      // (the derivative kernels'
 inline size_t linc_fx_smem(const DevMech& m) { return fx_smem(m.fxs[1], m.K, 256); }
 inline bool linc_fx_fits(const DevMech& m) { return m.fx_ok && m.fxs[1].np != 0 && linc_fx_smem(m) <= smem_limit(); }
 
-// 1/y for |y| in [2^-100, 2^100): the float reciprocal and two Newton steps (error near 2^-53)
+// 1/y for |y| in [2^-100, 2): the float reciprocal and two Newton steps (error near 2^-53)
 __device__ __forceinline__ double recip2(double y) {
     const double a = recip_nr(fabs(y)), r = fma(a, fma(-fabs(y), a, 1.0), a);
     return y < 0.0 ? -r : r;
 }
 
-// Points outside the form leave kFxSkip in their S1 slot for the marked pass of k_linc.cu.
+// Blocks with a point outside the form (the rates kernel's conditions, |Y_k| in [2^-100, 2)) leave
+// kFxSkip in their points' S1 slot for the marked pass of k_linc.cu.
 template <int NP, int OWN, int BLOCKS, bool OUT>
 __global__ void __launch_bounds__(32 * NP, BLOCKS)
     linc_fx_kernel(const DevMech m, const int64_t n, const int64_t ld, const double* __restrict__ T,
@@ -38,10 +39,6 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
     extern __shared__ __align__(16) unsigned char smem_fx[];
     const FxSet& f = m.fxs[1];
     unsigned char* im0 = smem_fx + kFxBase + kFxScalars * 256;
-    fx_image_load(f, 0, im0);
-    const FxTab ft = stage_fx_tables(reinterpret_cast<uint32_t*>(smem_fx), m.fx_tab);
-    const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem_fx + kFxTabBytes), m);
-    __syncthreads();
     const int K = m.K;
     const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
     const int64_t i0 = (int64_t)blockIdx.x * 32 + lane;
@@ -51,37 +48,52 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
     unsigned char* sP = im0 + 2 * f.image + lane * 8;
     unsigned char* sQ = sP + (size_t)(K + 1) * kFxDRow;
 
-    double Ti = T[i];
-    bool bad = !fx_T_ok(Ti);
-    if (bad) Ti = 1000.0;
+    // a block with a point outside the form leaves here, all its points marked (as in k_jvp_fx.cuh; one
+    // zero mass fraction in every block, 53 species, 262,144 points: 9.7 -> 6.8 ms)
+    const double Ti = T[i], pi = p[i];
     const unsigned long long Tb = (unsigned long long)__double_as_longlong(Ti);
+    double y[OWN];                                           // (all loads in flight at once)
+#pragma unroll
+    for (int j = 0; j < OWN; ++j) y[j] = part + NP * j < K ? Y[(int64_t)__ldg(&f.sp[part + NP * j].k) * ld + i] : 1.0;
+    fx_image_load(f, 0, im0);
+    const FxTab ft = stage_fx_tables(reinterpret_cast<uint32_t*>(smem_fx), m.fx_tab);
+    const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem_fx + kFxTabBytes), m);
+    bool bad = !fx_T_ok(Ti) || !fx_p_ok(pi);
+#pragma unroll
+    for (int j = 0; j < OWN; ++j) bad |= !fx_y_ok(y[j]);
+    if (__syncthreads_or(bad) != 0) {
+        if (part == 0 && live) lin[cs_S(m) * ldl + i] = __longlong_as_double((long long)kFxSkip);
+        fx_image_wait();
+        return;
+    }
     {
         unsigned long long z = 0, zc = 0;
-#pragma unroll 1
-        for (int k = part; k < K; k += NP) {
-            const FxSpecies* sp = f.sp + k;
-            const double y = Y[(int64_t)__ldg(&sp->k) * ld + i];
-            fx_add_fraction((unsigned long long)__double_as_longlong(y), __ldg((const long long*)&sp->w), z, zc, bad);
-            bad |= !log_range_ok(y);
+#pragma unroll
+        for (int j = 0; j < OWN; ++j) {
+            if (part + NP * j >= K) break;
+            fx_add_fraction((unsigned long long)__double_as_longlong(y[j]), __ldg((const long long*)&f.sp[part + NP * j].w), z, zc, bad);
         }
-        if (part == 0) bad |= !fx_point_scalars(m, Tb, p[i], sS, ft);
         reinterpret_cast<unsigned long long*>(sQ)[(2 * part) * 32] = z;
-        reinterpret_cast<unsigned long long*>(sQ)[(2 * part + 1) * 32] = bad ? kFxPoison : zc;
+        reinterpret_cast<unsigned long long*>(sQ)[(2 * part + 1) * 32] = zc;
     }
+    if (part == 0) fx_point_scalars(m, Tb, pi, sS, ft);
     __syncthreads();
     FxT P;
     P.lt = fx_frac63((unsigned long long)sS[kFxLT * 32] << 11);
     P.v = fx_frac63((unsigned long long)sS[kFxV * 32]);
-    bool good;
     {
         unsigned long long z = 0, zc = 0;
         for (int q = 0; q < NP; ++q) {
             z += reinterpret_cast<unsigned long long*>(sQ)[(2 * q) * 32];
             zc += reinterpret_cast<unsigned long long*>(sQ)[(2 * q + 1) * 32];
         }
-        good = !fx_sums_bad(z, zc);
-        const bool put = live && good;
-        const long long lrho = good ? sS[kFxLpRT * 32] - fx_log2_int(z, 60, ft) - m.fx_lmaxw : 0;
+        // (the conditions on the point sums)
+        if (__any_sync(0xffffffffu, fx_sums_bad(z, zc))) {
+            if (part == 0 && live) lin[cs_S(m) * ldl + i] = __longlong_as_double((long long)kFxSkip);
+            fx_image_wait();
+            return;
+        }
+        const long long lrho = sS[kFxLpRT * 32] - fx_log2_int(z, 60, ft) - m.fx_lmaxw;
         const FxFrac u = fx_frac_T(Tb);
 #pragma unroll 1
         for (int k = part; k < K; k += NP) {
@@ -90,13 +102,13 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             const double y = Y[(int64_t)ks * ld + i];
             unsigned char* row = sP + k * kFxDRow;
             const int64_t* c = fx_range(sp, Ti);
-            const long long a = good ? fx_log2_conc((unsigned long long)__double_as_longlong(y), __ldg((const long long*)&sp->lw) + lrho, ft) : 0;
+            const long long a = fx_log2_conc((unsigned long long)__double_as_longlong(y), __ldg((const long long*)&sp->lw) + lrho, ft);
             const long long h = fx_hRT(c, P, u);
             *reinterpret_cast<long long*>(row) = a;
             *reinterpret_cast<long long*>(row + kLcMu) = a + (fx_mu0(c, P, u) & ~1ll);
             *reinterpret_cast<long long*>(row + kLcE) = (1ll << kFxS) - h;
             *reinterpret_cast<long long*>(row + kLcCp) = fx_cpR(c, u);
-            if (put) {
+            if (live) {
                 lin[(cs_H(m) + ks) * ldl + i] = fx_to_d(h);
                 lin[(cs_iY(m) + ks) * ldl + i] = recip2(y);
                 lin[(cs_C(m) + ks) * ldl + i] = fx_exp2<true>(a, ft);
@@ -106,10 +118,9 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
 #pragma unroll
             for (int j = 0; j < kFxDRow / 256; ++j) *reinterpret_cast<long long*>(sP + K * kFxDRow + j * 256) = 0;
             sS[kFxLrho * 32] = lrho;
-            sS[kFxSum * 32] = good ? (long long)z : 0;
+            sS[kFxSum * 32] = (long long)z;
         }
     }
-    const bool store = live && good;
     fx_image_wait();
     __syncthreads();
 
@@ -199,7 +210,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             if (kind == 1 && zero) qq = qf = qr = 0.0;
             S1 = fma(qq, fx_to_d(Cp), S1);
             if constexpr (OUT) *reinterpret_cast<double*>(sQ + q * 256) = qq;
-            if (store) {
+            if (live) {
                 double* o = lin + i;
                 o[(int64_t)r * ldl] = fma(qq, aT, qr * fx_to_d(-E));
                 const int nu = __ldg(m.fx_nu1 + r);                  // first coefficients of the sides
@@ -232,7 +243,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             const unsigned char* row = sP + k * kFxDRow;
             const double o = *reinterpret_cast<const double*>(row);
             h = fma(fx_to_d((1ll << kFxS) - *reinterpret_cast<const long long*>(row + kLcE)), o, h);
-            if (store) omega[(int64_t)__ldg(&f.sp[k].k) * ld + i] = o;
+            if (live) omega[(int64_t)__ldg(&f.sp[k].k) * ld + i] = o;
         }
     }
     double* sR = reinterpret_cast<double*>(sQ);
@@ -244,9 +255,8 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
         S1 += sR[(2 * q) * 32];
         if constexpr (OUT) h += sR[(2 * q + 1) * 32];
     }
-    lin[cs_S(m) * ldl + i] = good ? S1 * kFxCpScale : __longlong_as_double((long long)kFxSkip);
-    if constexpr (OUT)
-        if (good) hrr[i] = -kR * Ti * h;
+    lin[cs_S(m) * ldl + i] = S1 * kFxCpScale;
+    if constexpr (OUT) hrr[i] = -kR * Ti * h;
 }
 
 template <bool OUT>

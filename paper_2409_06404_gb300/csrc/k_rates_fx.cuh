@@ -45,8 +45,8 @@ static __device__ __noinline__ float fx_troe_float(const TroeRecF* t, float Mf, 
 }
 
 // NP parts per point, 32 points per block.  RHS: the implicit-stage sources instead (omega ->
-// W_k omega_k / rho, hrr -> hrr/(rho c_p)).  A point outside the fixed-point form (fx_T_ok,
-// fx_add_fraction, fx_point_scalars, fx_sums_bad) leaves kFxSkip in its hrr: the fallback pass
+// W_k omega_k / rho, hrr -> hrr/(rho c_p)).  A point outside the fixed-point form (fx_T_ok, fx_p_ok,
+// fx_add_fraction, fx_sums_bad) leaves kFxSkip in its hrr: the fallback pass
 // (k_rates.cuh) takes it.
 // MIXED (NK_MIXED): ln k_f and the whole falloff in single precision, operation by operation as the
 // pair kernel's mixed form has them (so its results stay, to some 1e-13); concentrations, K_c, the
@@ -60,21 +60,29 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
     extern __shared__ __align__(16) unsigned char smem_fx[];
     unsigned char* im0 = smem_fx + kFxBase + kFxScalars * 256;
     const FxSet& f = m.fxs[0];
-    fx_image_load(f, 0, im0);
-    const FxTab ft = stage_fx_tables(reinterpret_cast<uint32_t*>(smem_fx), m.fx_tab);
-    const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem_fx + kFxTabBytes), m);   // (Troe)
-    __syncthreads();
     const int K = m.K;
     const int lane = threadIdx.x & 31, part = threadIdx.x >> 5;
     const int64_t i0 = (int64_t)blockIdx.x * 32 + lane;
     const bool live = i0 < n;
     const int64_t i = live ? i0 : n - 1;                 // idle lanes of the last block repeat point n-1
+    double Ti = T[i];
+    const double pi = p[i];
+    bool bad = !fx_T_ok(Ti) || !fx_p_ok(pi);
+    // A block with no point in T's and p's ranges leaves before its set-up (every part holds the same
+    // points).  Among others single points are left to the fallback pass alone: a point's result does
+    // not depend on its neighbours.
+    if (__all_sync(0xffffffffu, bad)) {
+        if (part == 0 && live) hrr[i] = __longlong_as_double((long long)kFxSkip);
+        return;
+    }
+    fx_image_load(f, 0, im0);
+    const FxTab ft = stage_fx_tables(reinterpret_cast<uint32_t*>(smem_fx), m.fx_tab);
+    const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem_fx + kFxTabBytes), m);   // (Troe)
+    __syncthreads();
     long long* sS = reinterpret_cast<long long*>(smem_fx + kFxBase) + lane;
     unsigned char* sP = im0 + 2 * f.image + lane * 8;                         // species rows
     unsigned char* sQ = sP + (size_t)(K + 1) * kFxRow;                           // rates of progress
 
-    double Ti = T[i];
-    bool bad = !fx_T_ok(Ti);
     if (bad) Ti = 1000.0;                                // the lane goes on with any state, its results are not stored
     const unsigned long long Tb = (unsigned long long)__double_as_longlong(Ti);
     {
@@ -85,7 +93,7 @@ __global__ void __launch_bounds__(32 * NP, NP <= 32 ? 32 / NP : 1)
             fx_add_fraction((unsigned long long)__double_as_longlong(Y[(int64_t)__ldg(&sp->k) * ld + i]),
                             __ldg((const long long*)&sp->w), z, zc, bad);
         }
-        if (part == 0) bad |= !fx_point_scalars(m, Tb, p[i], sS, ft);
+        if (part == 0) fx_point_scalars(m, Tb, pi, sS, ft);
         reinterpret_cast<unsigned long long*>(sQ)[(2 * part) * 32] = z;
         reinterpret_cast<unsigned long long*>(sQ)[(2 * part + 1) * 32] = bad ? kFxPoison : zc;
     }

@@ -25,8 +25,9 @@ inline size_t vjp_fx_smem(const DevMech& m, bool want_g) {
 }
 inline bool vjp_fx_fits(const DevMech& m) { return m.fx_ok && m.fxs[1].np != 0 && vjp_fx_smem(m, true) <= smem_limit(); }
 
-// Points outside the form (the rates kernel's conditions; Y_k and bar_omega_k in the pairs' range)
-// leave kFxSkip in gT for the marked passes of k_vjp.cu and add nothing to the ln A sums.
+// Tiles with a point outside the form (the rates kernel's conditions, |Y_k| in [2^-100, 2),
+// bar_omega_k in the pairs' range) leave kFxSkip in their points' gT for the marked passes of k_vjp.cu
+// and add nothing to the ln A sums.
 template <int NP, int OWN, int BLOCKS, bool WANT_G, bool HB>
 __global__ void __launch_bounds__(32 * NP, BLOCKS)
     vjp_fx_kernel(const DevMech m, const int64_t n, const int64_t ld, const double* __restrict__ T,
@@ -55,11 +56,10 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
         const int64_t i = live ? i0 : n - 1;
         __syncthreads();                                  // the tables; the last tile's sums are read
         fx_image_load(f, 0, im0);
-        double Ti = T[i];
-        bool bad = !fx_T_ok(Ti);
-        if (bad) Ti = 1000.0;
+        const double Ti = T[i], pi = p[i];
         const unsigned long long Tb = (unsigned long long)__double_as_longlong(Ti);
         {
+            bool bad = !fx_T_ok(Ti) || !fx_p_ok(pi);
             unsigned long long z = 0, zc = 0;
 #pragma unroll 1
             for (int k = part; k < K; k += NP) {
@@ -67,25 +67,35 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                 const int64_t at = (int64_t)__ldg(&sp->k) * ld + i;
                 const double y = Y[at];
                 fx_add_fraction((unsigned long long)__double_as_longlong(y), __ldg((const long long*)&sp->w), z, zc, bad);
-                bad |= !(log_range_ok(y) && pair_range_ok(bar_omega[at]));
+                bad |= !(fx_y_ok(y) && pair_range_ok(bar_omega[at]));
             }
-            if (part == 0) bad |= !fx_point_scalars(m, Tb, p[i], sS, ft);
+            if (part == 0) fx_point_scalars(m, Tb, pi, sS, ft);
             reinterpret_cast<unsigned long long*>(sQ)[(2 * part) * 32] = z;
-            reinterpret_cast<unsigned long long*>(sQ)[(2 * part + 1) * 32] = bad ? kFxPoison : zc;
+            reinterpret_cast<unsigned long long*>(sQ)[(2 * part + 1) * 32] = zc;
+            // a tile with a point outside the form is left to the marked passes, all its points marked
+            // (as in k_jvp_fx.cuh)
+            if (__syncthreads_or(bad) != 0) {
+                if (live && part == 0) gT[i] = __longlong_as_double((long long)kFxSkip);
+                fx_image_wait();
+                continue;
+            }
         }
-        __syncthreads();
         FxT P;
         P.lt = fx_frac63((unsigned long long)sS[kFxLT * 32] << 11);
         P.v = fx_frac63((unsigned long long)sS[kFxV * 32]);
-        bool good;
         {
             unsigned long long z = 0, zc = 0;
             for (int q = 0; q < NP; ++q) {
                 z += reinterpret_cast<unsigned long long*>(sQ)[(2 * q) * 32];
                 zc += reinterpret_cast<unsigned long long*>(sQ)[(2 * q + 1) * 32];
             }
-            good = !fx_sums_bad(z, zc);
-            const long long lrho = good ? sS[kFxLpRT * 32] - fx_log2_int(z, 60, ft) - m.fx_lmaxw : 0;
+            // (the conditions on the point sums)
+            if (__any_sync(0xffffffffu, fx_sums_bad(z, zc))) {
+                if (live && part == 0) gT[i] = __longlong_as_double((long long)kFxSkip);
+                fx_image_wait();
+                continue;
+            }
+            const long long lrho = sS[kFxLpRT * 32] - fx_log2_int(z, 60, ft) - m.fx_lmaxw;
             const FxFrac u = fx_frac_T(Tb);
 #pragma unroll 1
             for (int k = part; k < K; k += NP) {
@@ -93,8 +103,8 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                 const int64_t at = (int64_t)__ldg(&sp->k) * ld + i;
                 unsigned char* row = sP + k * kFxDRow;
                 const int64_t* c = fx_range(sp, Ti);
-                const long long a = good ? fx_log2_conc((unsigned long long)__double_as_longlong(Y[at]), __ldg((const long long*)&sp->lw) + lrho, ft) : 0;
-                const dfl w = good ? split_pair(bar_omega[at]) : dfl{0.0f, 0.0f};
+                const long long a = fx_log2_conc((unsigned long long)__double_as_longlong(Y[at]), __ldg((const long long*)&sp->lw) + lrho, ft);
+                const dfl w = split_pair(bar_omega[at]);
                 *reinterpret_cast<long long*>(row) = a;
                 *reinterpret_cast<long long*>(row + kVjMu) = a + (fx_mu0(c, P, u) & ~1ll);
                 *reinterpret_cast<float2*>(row + kVjW) = make_float2(w.h, w.l);
@@ -103,10 +113,9 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             }
             if (part == 0) {
                 sS[kFxLrho * 32] = lrho;
-                sS[kFxSum * 32] = good ? (long long)z : 0;
+                sS[kFxSum * 32] = (long long)z;
             }
         }
-        const bool valid = live && good;
         const double hbRT = HB ? bar_hrr[i] * (kR * Ti) : 0.0, hbCp = -hbRT * kFxCpScale;
         fx_image_wait();
         __syncthreads();
@@ -152,10 +161,10 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                         ws_ = df_add(ws_, df_neg(dfl_of(*reinterpret_cast<const float2*>(a + kVjW))));
                     }
                 }
-                double qbar = valid ? df_to_d(ws_) : 0.0;
+                double qbar = live ? df_to_d(ws_) : 0.0;
                 if constexpr (HB) {
                     const long long dH = ((long long)((info >> 4 & 15) - (info & 15)) << kFxS) - E;
-                    if (valid) qbar = fma(-hbRT, fx_to_d(dH), qbar);
+                    if (live) qbar = fma(-hbRT, fx_to_d(dH), qbar);
                 }
                 const long long ea = fx_mul(r1.x, P.v);  // -log2(e) Ea/RT
                 long long lnk = r0.x + fx_mul(r0.y, P.lt) + ea;
@@ -199,7 +208,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                     qf = fx_shift_edge(qf, d);
                     qr = fx_shift_edge(qr, d);
                 }
-                if (!valid) qf = qr = 0.0;
+                if (!live) qf = qr = 0.0;
                 const double F = qbar * qf, B = -qbar * qr;
                 const double G = F + B;
                 Tbar = fma(G, fx_to_d(s), Tbar);
@@ -208,7 +217,7 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
                 if (kind != 0) {
                     // X = G px rho'/[M] (z in units 2^(eff_shift - 60)); the p/(RT) part of [M]
                     double X = 0.0;
-                    if (z != 0 && valid) {
+                    if (z != 0 && live) {
                         const dfl iz = df_div(px, fx_to_pair(z < 0 ? -z : z));
                         X = G * (z < 0 ? -df_to_d(iz) : df_to_d(iz));                // times 2^-48 of z's unit
                     }
@@ -290,8 +299,8 @@ __global__ void __launch_bounds__(32 * NP, BLOCKS)
             Tbar += sR[(2 * q + 1) * 32];
         }
         // C_k = rho y_k, rho = p/(R T s), s = sum y_k: rho's cotangent through T and every Y_k
-        if (live && part == 0) gT[i] = good ? (Tbar - cc) / Ti : __longlong_as_double((long long)kFxSkip);
-        if (valid) {
+        if (live && part == 0) gT[i] = (Tbar - cc) / Ti;
+        if (live) {
             const double sbar = -cc * fx_exp2(sS[kFxLrho * 32] - sS[kFxLpRT * 32], ft);      // -cc/s
 #pragma unroll 1
             for (int k = part; k < K; k += NP) {

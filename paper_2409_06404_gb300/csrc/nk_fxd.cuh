@@ -43,10 +43,10 @@ __device__ __forceinline__ dfl split_pair_scaled(double v, int s) {
     const MantPair a = mant_pair(v);
     return a.e + s < -126 ? dfl{0.0f, 0.0f} : df_ldexp(a.m, a.e + s);
 }
-// |y| in [2^-100, 2^100)
-__device__ __forceinline__ bool log_range_ok(double y) {
+// |y| in [2^-100, 2): a mass fraction the derivative kernels take
+__device__ __forceinline__ bool fx_y_ok(double y) {
     const unsigned e = (unsigned)((unsigned long long)__double_as_longlong(y) >> 52) & 0x7ffu;
-    return e >= 1023u - 100u && e < 1023u + 100u;
+    return e - 923u <= 100u;
 }
 __device__ __forceinline__ dfl fxc_ln2() { return {0.693147182464599609375f, -1.9046542121259336e-09f}; }
 

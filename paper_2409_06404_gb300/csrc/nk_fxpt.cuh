@@ -108,6 +108,9 @@ __device__ __forceinline__ bool fx_T_ok(double T) {      // 128 (1 + 2^-31) < T 
     const long long b = __double_as_longlong(T);
     return b > 0x4060000000200000ll && b < 0x40afffffffc00000ll;
 }
+__device__ __forceinline__ bool fx_p_ok(double p) {      // [2^-100, 2^101)
+    return (unsigned)((unsigned long long)__double_as_longlong(p) >> 52) - 923u <= 200u;
+}
 // adds |y|'s part of sum |Y| (units 2^-40) and y/W's of sum Y/W (units 2^-60, relative to the
 // largest 1/W); bad: y is subnormal, 2 or more in magnitude, or not finite
 __device__ __forceinline__ void fx_add_fraction(unsigned long long yb, long long w, unsigned long long& z,
@@ -124,8 +127,8 @@ __device__ __forceinline__ void fx_add_fraction(unsigned long long yb, long long
 __device__ __forceinline__ bool fx_sums_bad(unsigned long long z, unsigned long long zc) {
     return zc > (3ull << 39) || z < (1ull << 50) || z > (1ull << 62);
 }
-// log2 T, 128/T and log2(p/(R T)) of a point into its scalars; false for p outside [2^-100, 2^101)
-__device__ __forceinline__ bool fx_point_scalars(const DevMech& m, unsigned long long Tb, double p, long long* sS,
+// log2 T, 128/T and log2(p/(R T)) of a point into its scalars
+__device__ __forceinline__ void fx_point_scalars(const DevMech& m, unsigned long long Tb, double p, long long* sS,
                                                  const FxTab& t) {
     const unsigned long long pb = (unsigned long long)__double_as_longlong(p);
     const unsigned long long vb = (unsigned long long)__double_as_longlong(128.0 / __longlong_as_double((long long)Tb));
@@ -133,7 +136,6 @@ __device__ __forceinline__ bool fx_point_scalars(const DevMech& m, unsigned long
     sS[kFxLT * 32] = lT;
     sS[kFxV * 32] = (long long)(((vb & 0x000fffffffffffffull) | 0x0010000000000000ull) << (((int)(vb >> 52) - 1012) & 63));
     sS[kFxLpRT * 32] = fx_log2_bits(pb, t) - m.fx_lR - lT;
-    return (unsigned)(pb >> 52) - 923u <= 200u;
 }
 // log2 |C_k| with the sign in bit 0, from the mass fraction's bits and log2(rho/W_k)
 __device__ __forceinline__ long long fx_log2_conc(unsigned long long yb, long long lr, const FxTab& t) {

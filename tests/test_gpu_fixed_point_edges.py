@@ -1,14 +1,15 @@
 """Edges of the fixed-point reaction kernels that ordinary fields do not reach: directions whose sums
-cancel.
+cancel, fields with points outside the form in some or all blocks.
 
 Tolerance 1e-10 of the cancellation-aware scales, as for every derivative kernel here."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import paper_2409_06404_gb300 as nk
 from paper_2409_06404_gb300 import synth
-from conftest import gpu_mechanism, to_dev, host, scaled_err
+from conftest import gpu_mechanism, to_dev, host, scaled_err, nu_matrix
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-10
@@ -36,3 +37,86 @@ def test_jvp_cancelling_colliders(cuda, K, R, d):
         for a, o, s in zip(got, want[:2], want[2:]):
             assert scaled_err(host(a), o, s) <= TOL
     m.close()
+
+
+@pytest.mark.parametrize("K,R", [(9, 21), (53, 120), (120, 200)])
+@pytest.mark.parametrize("where", ["all", "one", "warm"])
+def test_rejected_blocks(cuda, K, R, where):
+    """Zero mass fractions in every point, in one point of the second block, or (no zero) temperatures
+    above the form's in every point of the second block: all derivatives, with shifts of ln A."""
+    el = ("H", "O", "N") if K < 20 else ("C", "H", "O", "N")
+    mech = synth.make_mechanism(K, R, R // 6, R // 6, elements=el, seed=800 + K)
+    m = gpu_mechanism(mech)
+    n = 97
+    st = synth.states_uniform(K, n, seed=K)
+    T, p, Y = st.T.copy(), st.p.copy(), st.Y.copy()
+    if where == "warm":
+        T[32:64] = 4200.0
+    else:
+        Y[K // 2, slice(None) if where == "all" else 40] = 0.0
+    rng = np.random.default_rng(K)
+    vT, vY, wb, hb = rng.standard_normal(n), rng.standard_normal((K, n)), rng.standard_normal((K, n)), 1e-5 * rng.standard_normal(n)
+    dA = 0.1 * rng.standard_normal(R)
+    S, (vTt, vYt, wbt, hbt, dAt) = to_dev(T, p, Y), to_dev(vT, vY, wb, hb, dA)
+
+    dw, dh, dws, dhs = oracle.jvp(mech, T, p, Y, vT, vY, dlnA=dA, scales=True)
+    lin, w, h = nk.rates_linearize_compact(m, *S, dlnA=dAt, primal=True)
+    for a, b in (nk.rates_jvp(m, *S, vTt, vYt, dlnA=dAt), nk.rates_jvp_linearized_compact(m, *S, lin, vTt, vYt)):
+        assert scaled_err(host(a), dw, dws) <= TOL and scaled_err(host(b), dh, dhs) <= TOL
+    wo, ho, ws, hs = oracle.rates(mech, T, p, Y, dlnA=dA, scales=True)
+    assert scaled_err(host(w), wo, ws) <= TOL and scaled_err(host(h), ho, hs) <= TOL
+    for a, o, s in zip(nk.rhs_jvp(m, *S, vTt, vYt), *[oracle.rhs_jvp(mech, T, p, Y, vT, vY, scales=True)[i:i + 2] for i in (0, 2)]):
+        assert scaled_err(host(a), o, s) <= TOL
+
+    gT, gY, g = nk.rates_vjp(m, *S, wbt, hbt, dlnA=dAt)
+    J, Js = oracle.jacobian(mech, T, p, Y, dlnA=dA, scales=True)
+    u = np.vstack([wb, hb[None]])
+    JTu, scale = np.einsum("nij,in->jn", J, u), np.einsum("nij,in->jn", Js, np.abs(u))
+    assert scaled_err(host(gT), JTu[0], scale[0]) <= TOL and scaled_err(host(gY), JTu[1:], scale[1:]) <= TOL
+    fwd, rev = oracle.rates_of_progress(mech, T, p, Y, dlnA=dA)
+    qbar = np.abs(nu_matrix(mech)).T @ (np.abs(wb) + np.abs(hb * oracle.thermo(mech, T, p, Y)["h_k"]))
+    assert scaled_err(host(g), oracle.grad_lnA(mech, T, p, Y, wb, hb, dlnA=dA), np.sum(qbar * (fwd + rev), axis=1)) <= TOL
+    m.close()
+
+
+def _median_ms(f):
+    f()
+    t = []
+    for _ in range(9):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        t.append(a.elapsed_time(b))
+    return sorted(t)[len(t) // 2]
+
+
+def _pair_only(mech):
+    """The same mechanism with five molecules on a side of one reaction, which keeps it off the
+    fixed-point kernels."""
+    other = mech.copy()
+    other.reac_nu[0] = 5
+    return other
+
+
+@pytest.mark.parametrize("name", ["h2_9sp_21rx", "ch4_53sp_325rx"])
+@pytest.mark.parametrize("call", ["jvp", "rhs_jvp", "linearize"])
+def test_rejected_blocks_cost_one_pass(cuda, name, call):
+    """Fields all of whose blocks hold a point outside the form take the pair kernels' time: at most
+    1.2 of what a mechanism that never enters the fixed-point kernels takes (the set-up that finds
+    the points out is about a twentieth of a pass; a whole fixed-point pass is half of one)."""
+    mech = synth.mechanism(name)
+    n = 65536
+    st = synth.states_uniform(mech.K, n, seed=2)
+    st.Y[3, ::32] = 0.0
+    T, p, Y = to_dev(st.T, st.p, st.Y)
+    vT, vY = torch.randn_like(T), torch.randn_like(Y)
+    ms = []
+    for mm in (mech, _pair_only(mech)):
+        m = gpu_mechanism(mm)
+        lin = torch.empty((nk.linearization_slots_compact(m), n), dtype=torch.float64, device="cuda")
+        ms.append(_median_ms({"jvp": lambda: nk.rates_jvp(m, T, p, Y, vT, vY), "rhs_jvp": lambda: nk.rhs_jvp(m, T, p, Y, vT, vY),
+                              "linearize": lambda: nk.rates_linearize_compact(m, T, p, Y, lin=lin, primal=True)}[call]))
+        m.close()
+    assert ms[0] <= 1.2 * ms[1], ms
