@@ -359,10 +359,14 @@ __host__ __device__ constexpr int shared_rows() {
 //
 // RHS: write the implicit-stage sources instead: omega -> W_k omega_k / rho, hrr -> hrr/(rho c_p).
 //
-// PASS 2 (kDF, kMixed): as 1 for the points whose hrr holds kFxSkip, whatever their state.  PASS (kDF and kMixed): 0 takes the blocks without a negative concentration and skips the
+// PASS (kDF and kMixed): 0 takes the blocks without a negative concentration and skips the
 // others, 1 takes only those, with the concentrations' signs in a byte row after the omega_k row
 // (rates_smem_signs); so the common pass carries no sign work.  The second pass leaves at once
-// where no mass fraction of the block is negative.  The native form has one pass (0) over every
+// where no mass fraction of the block is negative.  PASS 2: the points whose hrr holds kFxSkip, left by
+// the fixed-point kernel (k_rates_fx.cuh), whatever their state; a block without a negative
+// concentration takes pass 0's rounds there, one launch being all that an ordinary field should pay
+// (a field above 4096 K, 53 species, 262,144 points: 5.01 ms with the fixed-point pass made all the
+// same and 4 parts a point -> 2.97; 9 species: 0.63 -> 0.29).  The native form has one pass (0) over every
 // block.
 template <int BLK, int NP, int PREC, bool RHS, int PASS>
 __global__ void __launch_bounds__(BLK * NP, (PREC != kNative ? 768 : 640) / (BLK * NP))
@@ -451,17 +455,24 @@ __global__ void __launch_bounds__(BLK * NP, (PREC != kNative ? 768 : 640) / (BLK
         if (PASS == 0 ? vote : !vote) return;     // the other pass takes this block
     }
 
-    if constexpr (NP == 1) {
-        const int e1 = m.R_el, t1 = m.R_el + m.R_tb;
-        reaction_group<BLK, PREC, 0, SG>(m, 0, e1, sC, sG, sW, sg, P, dlnA, mt, dt);
-        reaction_group<BLK, PREC, 1, SG>(m, e1, t1, sC, sG, sW, sg, P, dlnA, mt, dt);
-        reaction_group<BLK, PREC, 2, SG>(m, t1, m.R, sC, sG, sW, sg, P, dlnA, mt, dt);
-    } else {
-        // (each round ends with a barrier: the omega_k row is complete after the last one)
-        reaction_rounds<BLK, NP, PREC, 0, SG>(m, part, sC, sG, sW, sg, P, dlnA, mt, dt);
-        reaction_rounds<BLK, NP, PREC, 1, SG>(m, part, sC, sG, sW, sg, P, dlnA, mt, dt);
-        reaction_rounds<BLK, NP, PREC, 2, SG>(m, part, sC, sG, sW, sg, P, dlnA, mt, dt);
-    }
+    auto reactions = [&](auto with_signs) {
+        constexpr bool S = decltype(with_signs)::value;
+        if constexpr (NP == 1) {
+            const int e1 = m.R_el, t1 = m.R_el + m.R_tb;
+            reaction_group<BLK, PREC, 0, S>(m, 0, e1, sC, sG, sW, sg, P, dlnA, mt, dt);
+            reaction_group<BLK, PREC, 1, S>(m, e1, t1, sC, sG, sW, sg, P, dlnA, mt, dt);
+            reaction_group<BLK, PREC, 2, S>(m, t1, m.R, sC, sG, sW, sg, P, dlnA, mt, dt);
+        } else {
+            // (each round ends with a barrier: the omega_k row is complete after the last one)
+            reaction_rounds<BLK, NP, PREC, 0, S>(m, part, sC, sG, sW, sg, P, dlnA, mt, dt);
+            reaction_rounds<BLK, NP, PREC, 1, S>(m, part, sC, sG, sW, sg, P, dlnA, mt, dt);
+            reaction_rounds<BLK, NP, PREC, 2, S>(m, part, sC, sG, sW, sg, P, dlnA, mt, dt);
+        }
+    };
+    if (PASS == 2 && !vote)
+        reactions(std::false_type{});
+    else
+        reactions(std::bool_constant<SG>{});
 
     // omega_k (or the source W_k omega_k / rho), sum_k h_k/RT omega_k and, for the sources,
     // c_p/R = sum_k Y_k/W_k c_p,k/R of this part's species
@@ -555,21 +566,6 @@ cudaError_t launch_idx(int idx, std::integer_sequence<int, S...>, const DevMech&
     return e;
 }
 
-
-// The points that the fixed-point kernel (k_rates_fx.cuh) left marked in hrr, in the kDF or
-// kMixed form with signs (any state).
-template <int PREC, bool RHS>
-cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
-                          const double* dlnA, double* omega, double* hrr, cudaStream_t st) {
-    const Shape sh{32, m.K >= 8 ? 4 : 1};
-    const size_t smem = rates_smem<PREC>(m.K, sh) + rates_smem_signs(m.K, sh);
-    auto kern = sh.np == 4 ? rates_kernel<32, 4, PREC, RHS, 2> : rates_kernel<32, 1, PREC, RHS, 2>;
-    const cudaError_t e = ensure_smem((const void*)kern, smem);
-    if (e != cudaSuccess) return e;
-    kern<<<(unsigned)((n + 31) / 32), 32 * sh.np, smem, st>>>(m, n, ld, T, p, Y, dlnA, omega, hrr);
-    return cudaGetLastError();
-}
-
 // The shape with the most resident warps per SM (CUDA's occupancy calculator: shared memory,
 // registers, threads), fewer parts on ties.  Cached per
 // (device, K, form).
@@ -613,6 +609,35 @@ int plan_shape(int K) {
         g_plans.push_back({dev, K, PREC, (int)RHS, best});
     }
     return best;
+}
+
+// The points that the fixed-point kernel (k_rates_fx.cuh) left marked in hrr, in the kDF or kMixed form's
+// shape.
+template <int PREC, bool RHS, int... S>
+cudaError_t launch_marked_idx(int idx, std::integer_sequence<int, S...>, const DevMech& m, int64_t n, int64_t ld,
+                              const double* T, const double* p, const double* Y, const double* dlnA, double* omega,
+                              double* hrr, cudaStream_t st) {
+    cudaError_t e = cudaErrorInvalidConfiguration;
+    ((S == idx ? (void)(e = [&] {
+        constexpr Shape sh = kShapes[S];
+        auto kern = kernel_of<PREC, RHS, S, 2>();
+        const size_t smem = rates_smem<PREC>(m.K, sh) + rates_smem_signs(m.K, sh);
+        const cudaError_t r = ensure_smem((const void*)kern, smem);
+        if (r != cudaSuccess) return r;
+        kern<<<(unsigned)((n + sh.blk - 1) / sh.blk), sh.blk * sh.np, smem, st>>>(m, n, ld, T, p, Y, dlnA, omega, hrr);
+        return cudaGetLastError();
+    }())
+               : (void)0),
+     ...);
+    return e;
+}
+template <int PREC, bool RHS>
+cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
+                          const double* dlnA, double* omega, double* hrr, cudaStream_t st) {
+    const int idx = plan_shape<PREC, RHS>(m.K);
+    if (idx < 0) return cudaErrorInvalidConfiguration;
+    return launch_marked_idx<PREC, RHS>(idx, std::make_integer_sequence<int, kNumShapes>{}, m, n, ld, T, p, Y, dlnA,
+                                        omega, hrr, st);
 }
 
 template <int PREC, bool RHS>

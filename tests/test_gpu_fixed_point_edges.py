@@ -120,3 +120,20 @@ def test_rejected_blocks_cost_one_pass(cuda, name, call):
                               "linearize": lambda: nk.rates_linearize_compact(m, T, p, Y, lin=lin, primal=True)}[call]))
         m.close()
     assert ms[0] <= 1.2 * ms[1], ms
+
+
+@pytest.mark.parametrize("name", ["h2_9sp_21rx", "ch4_53sp_325rx"])
+@pytest.mark.parametrize("T0", [110.0, 4500.0])
+def test_rates_out_of_range_cost_one_pass(cuda, name, T0):
+    """Rates and sources of fields wholly outside 128 .. 4096 K: as the derivatives above."""
+    mech = synth.mechanism(name)
+    n = 131072
+    st = synth.states_uniform(mech.K, n, seed=2)
+    _, p, Y = to_dev(st.T, st.p, st.Y)
+    T = torch.full_like(p, T0)
+    ms = []
+    for mm in (mech, _pair_only(mech)):
+        m = gpu_mechanism(mm)
+        ms.append([_median_ms(lambda: nk.rates_eval(m, T, p, Y)), _median_ms(lambda: nk.rhs_eval(m, T, p, Y, precision="mixed"))])
+        m.close()
+    assert ms[0][0] <= 1.2 * ms[1][0] and ms[0][1] <= 1.2 * ms[1][1], ms
