@@ -470,7 +470,8 @@ size_t vjp_smem(int K, int R, int mslots, bool want_g) {
 // PASS 0 takes the tiles of the logarithmic form and skips the others; PASS 1 takes only those
 // (products in double).  Each pass alone compiles to fewer registers than both paths together:
 // the logarithmic pass runs four blocks of 4 warps per SM, the fallback pass three.
-// MARKED: only the points whose gT holds kFxSkip (left by k_vjp_fx.cuh, which takes the others).
+// MARKED: only the points whose gT holds kFxSkip (left by k_vjp_fx.cuh, which takes the others); the
+// ln A sums are added to the first `have` rows of ws, which the kernels before it on the stream wrote.
 template <int NP, bool WANT_G, bool HB, int PASS, bool MARKED = false>
 __global__ void __launch_bounds__(kVjpBlk * NP, (PASS == 0 ? 512 : 384) / (kVjpBlk * NP)) vjp_kernel(const DevMech m, const int64_t n, const int64_t ld,
                                                            const double* __restrict__ T, const double* __restrict__ p,
@@ -479,7 +480,7 @@ __global__ void __launch_bounds__(kVjpBlk * NP, (PASS == 0 ? 512 : 384) / (kVjpB
                                                            const double* __restrict__ bar_omega,
                                                            const double* __restrict__ bar_hrr,
                                                            double* __restrict__ gT, double* __restrict__ gY,
-                                                           double* __restrict__ ws) {
+                                                           double* __restrict__ ws, const int64_t have) {
     constexpr int BLK = kVjpBlk, NT = BLK * NP;
     extern __shared__ double smem[];
     const DfTab dt = stage_df_tables(reinterpret_cast<float2*>(smem), m);
@@ -602,8 +603,11 @@ __global__ void __launch_bounds__(kVjpBlk * NP, (PASS == 0 ? 512 : 384) / (kVjpB
         __syncthreads();                                          // before the next tile reuses the rows
     }
 
-    if (WANT_G)
-        for (int r = threadIdx.x; r < R; r += NT) ws[(size_t)blockIdx.x * R + r] = gw[r];
+    if (WANT_G) {
+        double* row = ws + (size_t)blockIdx.x * R;
+        const bool add = MARKED && blockIdx.x < have;
+        for (int r = threadIdx.x; r < R; r += NT) row[r] = add ? row[r] + gw[r] : gw[r];
+    }
 }
 
 // g[orig(r)] = sum over blocks of ws[b][r], blocks in order
@@ -637,6 +641,7 @@ struct VjpPlan {
     int parts_idx[2];   // index into kParts, per pass
     int grid_cap[2];    // blocks of each pass
     int fx_cap;         // blocks of the fixed-point kernel (0: it does not take the mechanism)
+    int marked_cap;     // blocks of each pass behind it
 };
 std::mutex g_plan_mu;
 std::vector<VjpPlan> g_plans;
@@ -685,12 +690,11 @@ bool plan_variant(const DevMech& m, VjpPlan& out) {
     int p0 = -1, p1 = -1, b0 = 0, b1 = 0;
     if (!plan_pass<WANT_G, HB, 0>(m, sms, per_block, p0, b0)) return false;
     if (!plan_pass<WANT_G, HB, 1>(m, sms, per_block, p1, b1)) return false;
-    out = VjpPlan{dev, m.K, m.R, m.mslots2, m.mslots4, variant, {p0, p1}, {sms * b0, sms * b1}, 0};
-    // with the fixed-point kernel the two passes see only marked points: half a block per SM each,
-    // so that the partial sums' rows stay no more than without it (b0 + b1 blocks per SM)
+    out = VjpPlan{dev, m.K, m.R, m.mslots2, m.mslots4, variant, {p0, p1}, {sms * b0, sms * b1}, 0, 0};
+    // with the fixed-point kernel the two passes see only marked points
     if (vjp_fx_fits(m)) {
-        out.fx_cap = sms * std::min(vjp_fx_blocks(m), std::max(1, b0 + b1 - 1));
-        out.grid_cap[0] = out.grid_cap[1] = std::max(1, sms / 2);
+        out.fx_cap = sms * std::min(vjp_fx_blocks(m), b0 + b1);
+        out.marked_cap = std::max(1, sms / 2);
     }
     std::lock_guard<std::mutex> lk(g_plan_mu);
     g_plans.push_back(out);
@@ -712,32 +716,42 @@ int64_t vjp_fx_grid(const VjpPlan& pl, int64_t n) {
     return tiles < pl.fx_cap ? tiles : pl.fx_cap;
 }
 
-// blocks of both passes and of the fixed-point kernel before them, the ln A partial sums' rows in
-// the workspace
-int64_t vjp_blocks(const VjpPlan& pl, int64_t n) { return vjp_fx_grid(pl, n) + vjp_grid(pl, 0, n) + vjp_grid(pl, 1, n); }
+int64_t vjp_marked_grid(const VjpPlan& pl, int64_t n) {
+    const int64_t tiles = (n + kVjpBlk - 1) / kVjpBlk;
+    return tiles < pl.marked_cap ? tiles : pl.marked_cap;
+}
+
+// The ln A partial sums' rows in the workspace: one per block of the two passes.
+int64_t vjp_rows(const VjpPlan& pl, int64_t n) { return vjp_grid(pl, 0, n) + vjp_grid(pl, 1, n); }
+
+// The rows that a call writes.  Behind the fixed-point kernel the passes add to its rows, so that the
+// workspace needs no more rows than the two passes alone (fx_cap is at most the sum of their caps).
+int64_t vjp_rows_used(const VjpPlan& pl, int64_t n) {
+    return pl.fx_cap ? std::max(vjp_fx_grid(pl, n), vjp_marked_grid(pl, n)) : vjp_rows(pl, n);
+}
 
 template <bool WANT_G, bool HB, int PASS, bool MARKED = false>
 cudaError_t launch_pass(const VjpPlan& pl, const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                         const double* Y, const double* dlnA, const double* bar_omega, const double* bar_hrr,
-                        double* gT, double* gY, double* ws, cudaStream_t s) {
+                        double* gT, double* gY, double* ws, int64_t have, cudaStream_t s) {
     const int np = kParts[pl.parts_idx[PASS]];
     const size_t smem = vjp_smem(m.K, m.R, vjp_mslots(m, np), WANT_G);
     const void* kp = kernel_ptr<WANT_G, HB, PASS, MARKED>(pl.parts_idx[PASS]);
     cudaError_t e = ensure_smem(kp, smem);
     if (e != cudaSuccess) return e;
-    const unsigned grid = (unsigned)vjp_grid(pl, PASS, n);
+    const unsigned grid = (unsigned)(MARKED ? vjp_marked_grid(pl, n) : vjp_grid(pl, PASS, n));
     switch (np) {
         case 1:
             vjp_kernel<1, WANT_G, HB, PASS, MARKED><<<grid, kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr,
-                                                                        gT, gY, ws);
+                                                                                gT, gY, ws, have);
             break;
         case 2:
             vjp_kernel<2, WANT_G, HB, PASS, MARKED><<<grid, 2 * kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega,
-                                                                            bar_hrr, gT, gY, ws);
+                                                                                    bar_hrr, gT, gY, ws, have);
             break;
         default:
             vjp_kernel<4, WANT_G, HB, PASS, MARKED><<<grid, 4 * kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega,
-                                                                            bar_hrr, gT, gY, ws);
+                                                                                    bar_hrr, gT, gY, ws, have);
     }
     return cudaGetLastError();
 }
@@ -747,19 +761,18 @@ cudaError_t launch_v(const VjpPlan& pl, const DevMech& m, int64_t n, int64_t ld,
                      const double* Y, const double* dlnA, const double* bar_omega, const double* bar_hrr, double* gT,
                      double* gY, double* ws, cudaStream_t s) {
     if (pl.fx_cap) {
-        const int64_t g = vjp_fx_grid(pl, n), g0 = vjp_grid(pl, 0, n);
+        const int64_t g = vjp_fx_grid(pl, n);
         cudaError_t e = launch_vjp_fx<WANT_G, HB>(m, g, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, s);
         if (e != cudaSuccess) return e;
-        e = launch_pass<WANT_G, HB, 0, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY,
-                                             ws ? ws + (size_t)g * m.R : nullptr, s);
+        e = launch_pass<WANT_G, HB, 0, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, g, s);
         if (e != cudaSuccess) return e;
-        return launch_pass<WANT_G, HB, 1, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY,
-                                                ws ? ws + (size_t)(g + g0) * m.R : nullptr, s);
+        return launch_pass<WANT_G, HB, 1, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws,
+                                                std::max(g, vjp_marked_grid(pl, n)), s);
     }
-    cudaError_t e = launch_pass<WANT_G, HB, 0>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, s);
+    cudaError_t e = launch_pass<WANT_G, HB, 0>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, 0, s);
     if (e != cudaSuccess) return e;
     double* ws1 = ws ? ws + (size_t)vjp_grid(pl, 0, n) * m.R : nullptr;
-    return launch_pass<WANT_G, HB, 1>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws1, s);
+    return launch_pass<WANT_G, HB, 1>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws1, 0, s);
 }
 
 }  // namespace
@@ -800,7 +813,7 @@ size_t vjp_workspace_bytes(const DevMech& m, int64_t n) {
     if (!plan_for(m, true, false, pl)) return 0;
     VjpPlan pl2;
     if (!plan_for(m, true, true, pl2)) return 0;
-    const int64_t blocks = std::max(vjp_blocks(pl, n), vjp_blocks(pl2, n));   // either cotangent set
+    const int64_t blocks = std::max(vjp_rows(pl, n), vjp_rows(pl2, n));   // either cotangent set
     return (size_t)blocks * m.R * sizeof(double);
 }
 
@@ -820,7 +833,7 @@ cudaError_t launch_vjp(const DevMech& m, int64_t n, int64_t ld, const double* T,
         e = hb ? launch_v<false, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, nullptr, s)
                : launch_v<false, false>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, nullptr, s);
     if (e != cudaSuccess || !want_g) return e;
-    reduce_blocks_kernel<<<(m.R + 127) / 128, 128, 0, s>>>(wsd, (int)vjp_blocks(pl, n), m.rxn, m.R, g_lnA);
+    reduce_blocks_kernel<<<(m.R + 127) / 128, 128, 0, s>>>(wsd, (int)vjp_rows_used(pl, n), m.rxn, m.R, g_lnA);
     return cudaGetLastError();
 }
 

@@ -137,3 +137,29 @@ def test_rates_out_of_range_cost_one_pass(cuda, name, T0):
         ms.append([_median_ms(lambda: nk.rates_eval(m, T, p, Y)), _median_ms(lambda: nk.rhs_eval(m, T, p, Y, precision="mixed"))])
         m.close()
     assert ms[0][0] <= 1.2 * ms[1][0] and ms[0][1] <= 1.2 * ms[1][1], ms
+
+
+def test_noalloc_vjp_takes_two_rows_a_tile(cuda):
+    """ln A partial sums take two rows of R per tile of 32 points: 2,000 points of 8,192 reactions fit
+    the 8 MiB scratch.  Points of each of the VJP's three kernels share the rows."""
+    mech = synth.make_mechanism(K=40, R=8192, n_tb=40, n_troe=40, seed=78)
+    m = gpu_mechanism(mech)
+    n = 2000
+    assert nk.rates_vjp_workspace(m, n) == 2 * 63 * mech.R * 8
+    st = synth.states_uniform(mech.K, n, seed=4)
+    T, Y = st.T.copy(), st.Y.copy()
+    T[320:640] = 4300.0
+    Y[5, 640:960] = 0.0
+    w = synth.normal((mech.K, n), 5)
+    Tt, pt, Yt, wt = to_dev(T, st.p, Y, w)
+    gT, gY, g1 = nk.rates_vjp(m, Tt, pt, Yt, wt)
+    gT2, gY2, g2 = torch.empty_like(gT), torch.empty_like(gY), torch.empty_like(g1)
+    P = lambda t: t.data_ptr()                                                                # noqa: E731
+    status = nk.lib().nk_rates_vjp_noalloc(m.handle, n, n, P(Tt), P(pt), P(Yt), None, P(wt), None, P(gT2), P(gY2), P(g2), None)
+    assert status == 0, nk.lib().nk_last_error()
+    torch.cuda.synchronize()
+    assert torch.equal(gT, gT2) and torch.equal(gY, gY2) and torch.equal(g1, g2)
+    fwd, rev = oracle.rates_of_progress(mech, T, st.p, Y)
+    scale = np.sum((np.abs(nu_matrix(mech)).T @ np.abs(w)) * (fwd + rev), axis=1)
+    assert scaled_err(host(g1), oracle.grad_lnA(mech, T, st.p, Y, w), scale) <= TOL
+    m.close()
