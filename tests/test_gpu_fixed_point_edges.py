@@ -101,7 +101,7 @@ def _pair_only(mech):
 
 
 @pytest.mark.parametrize("name", ["h2_9sp_21rx", "ch4_53sp_325rx"])
-@pytest.mark.parametrize("call", ["jvp", "rhs_jvp", "linearize"])
+@pytest.mark.parametrize("call", ["jvp", "rhs_jvp", "linearize", "vjp"])
 def test_rejected_blocks_cost_one_pass(cuda, name, call):
     """Fields all of whose blocks hold a point outside the form take the pair kernels' time: at most
     1.2 of what a mechanism that never enters the fixed-point kernels takes (the set-up that finds
@@ -117,6 +117,7 @@ def test_rejected_blocks_cost_one_pass(cuda, name, call):
         m = gpu_mechanism(mm)
         lin = torch.empty((nk.linearization_slots_compact(m), n), dtype=torch.float64, device="cuda")
         ms.append(_median_ms({"jvp": lambda: nk.rates_jvp(m, T, p, Y, vT, vY), "rhs_jvp": lambda: nk.rhs_jvp(m, T, p, Y, vT, vY),
+                              "vjp": lambda: nk.rates_vjp(m, T, p, Y, vY, vT),
                               "linearize": lambda: nk.rates_linearize_compact(m, T, p, Y, lin=lin, primal=True)}[call]))
         m.close()
     assert ms[0] <= 1.2 * ms[1], ms
