@@ -9,7 +9,7 @@
 // 3K + 2K + 2 and writes 3K + 6 doubles per point.  The FP64 pipe bounds it: 15 operations per
 // species and point; c_p,k comes from integer polynomials (nk_thermo.cuh) for 64 K <= T < 4096 K,
 // with it in doubles it took 23.  (Keeping a_k in shared memory between the passes saves one more
-// but holds the SM at 16 warps.)  With the thermodynamics, 53 species, 884,736 points: 4.05 -> 2.12 ms
+// but holds the SM at 16 warps.)  With the thermodynamics, 53 species, 884,736 points: 4.05 -> 2.08 ms
 // (3.09 with 64 threads and the shared array).
 #include "nk_thermo.cuh"
 
@@ -17,6 +17,44 @@ namespace nk {
 namespace {
 
 constexpr int kBlk = 128;
+
+// c_p,k of the enthalpy flux: not wanted, from the integer polynomials, in doubles.  A loop of its own
+// for each, so that it unrolls and loads four species ahead: with the choice inside the loop a thread waited
+// for one species' loads at a time, which bounds fields below some 200,000 points (53 species, 5,000 points:
+// 90.6 -> 51.6 us, without the enthalpy flux 59.9 -> 33.3; 40,000: 170 -> 104; 884,736: 1.53 -> 1.46 ms).
+enum { kNoFlux, kIntCp, kDoubleCp };
+
+// The second pass: j_k, and sum_k c_p,k j_k (J/(kg K)) for the enthalpy flux.
+template <int CP>
+__device__ __forceinline__ void flux_pass(const DevMech& m, int64_t ld, int64_t i, double Ti, const ThT& t, double c0,
+                                          double S0, double S1, double S2, const double* __restrict__ Y,
+                                          const double* __restrict__ D, const double* __restrict__ G,
+                                          double* __restrict__ j, double& h0, double& h1, double& h2) {
+    const int64_t cs = (int64_t)m.K * ld;
+#pragma unroll 4
+    for (int k = 0; k < m.K; ++k) {
+        const int64_t o = (int64_t)k * ld + i;
+        const double a = c0 * (__ldg(m.W + k) * D[o]), y = Y[o];
+        const double j0 = fma(a, G[o], -y * S0), j1 = fma(a, G[o + cs], -y * S1), j2 = fma(a, G[o + 2 * cs], -y * S2);
+        j[o] = j0;
+        j[o + cs] = j1;
+        j[o + 2 * cs] = j2;
+        if constexpr (CP != kNoFlux) {
+            double cpk;
+            if constexpr (CP == kIntCp) {
+                const FxThermo* x = m.th + k;
+                const double2 head = __ldg(reinterpret_cast<const double2*>(x));
+                const bool lo = __double_as_longlong(Ti) <= __double_as_longlong(head.x);
+                cpk = th_cp(lo ? x->c[0] : x->c[1], lo ? t.lo : t.hi, __double2loint(head.y)) * __ldg(m.invW + k);
+            } else {
+                cpk = kR * nasa_cpR(nasa_range(m, k, Ti), Ti) * __ldg(m.invW + k);
+            }
+            h0 = fma(cpk, j0, h0);
+            h1 = fma(cpk, j1, h1);
+            h2 = fma(cpk, j2, h2);
+        }
+    }
+}
 
 __global__ void __launch_bounds__(kBlk) diffusion_kernel(const DevMech m, const int64_t n, const int64_t ld,
                                                          const double* __restrict__ T, const double* __restrict__ p,
@@ -29,6 +67,7 @@ __global__ void __launch_bounds__(kBlk) diffusion_kernel(const DevMech m, const 
     const int64_t cs = (int64_t)K * ld;                       // component stride of grad X and j
     const double Ti = T[i];
     double s = 0.0, S0 = 0.0, S1 = 0.0, S2 = 0.0;
+#pragma unroll 4
     for (int k = 0; k < K; ++k) {
         const int64_t o = (int64_t)k * ld + i;
         s = fma(Y[o], __ldg(m.invW + k), s);
@@ -50,33 +89,17 @@ __global__ void __launch_bounds__(kBlk) diffusion_kernel(const DevMech m, const 
     }
     const ThT t = th_fractions(m, Ti, 8.0);                   // (no logarithm needed)
     double h0 = 0.0, h1 = 0.0, h2 = 0.0;
-    for (int k = 0; k < K; ++k) {
-        const int64_t o = (int64_t)k * ld + i;
-        const double a = c0 * (__ldg(m.W + k) * D[o]), y = Y[o];
-        const double j0 = fma(a, G[o], -y * S0), j1 = fma(a, G[o + cs], -y * S1), j2 = fma(a, G[o + 2 * cs], -y * S2);
-        j[o] = j0;
-        j[o + cs] = j1;
-        j[o + 2 * cs] = j2;
-        if (hf) {
-            double cpk;                                       // J/(kg K)
-            if (t.ok) {
-                const FxThermo* x = m.th + k;
-                const double2 head = __ldg(reinterpret_cast<const double2*>(x));
-                const bool lo = __double_as_longlong(Ti) <= __double_as_longlong(head.x);
-                cpk = th_cp(lo ? x->c[0] : x->c[1], lo ? t.lo : t.hi, __double2loint(head.y)) * __ldg(m.invW + k);
-            } else {
-                cpk = kR * nasa_cpR(nasa_range(m, k, Ti), Ti) * __ldg(m.invW + k);
-            }
-            h0 = fma(cpk, j0, h0);
-            h1 = fma(cpk, j1, h1);
-            h2 = fma(cpk, j2, h2);
-        }
+    if (!hf) {
+        flux_pass<kNoFlux>(m, ld, i, Ti, t, c0, S0, S1, S2, Y, D, G, j, h0, h1, h2);
+        return;
     }
-    if (hf) {
-        hf[i] = h0;
-        hf[ld + i] = h1;
-        hf[2 * ld + i] = h2;
-    }
+    if (t.ok)
+        flux_pass<kIntCp>(m, ld, i, Ti, t, c0, S0, S1, S2, Y, D, G, j, h0, h1, h2);
+    else
+        flux_pass<kDoubleCp>(m, ld, i, Ti, t, c0, S0, S1, S2, Y, D, G, j, h0, h1, h2);
+    hf[i] = h0;
+    hf[ld + i] = h1;
+    hf[2 * ld + i] = h2;
 }
 
 }  // namespace

@@ -164,3 +164,18 @@ def test_noalloc_vjp_takes_two_rows_a_tile(cuda):
     scale = np.sum((np.abs(nu_matrix(mech)).T @ np.abs(w)) * (fwd + rev), axis=1)
     assert scaled_err(host(g1), oracle.grad_lnA(mech, T, st.p, Y, w), scale) <= TOL
     m.close()
+
+
+def test_fluxes_of_few_points(cuda):
+    """Few points: thermodynamics and diffusion fluxes both wait for one pass of loads per species, the
+    fluxes for a second pass of loads that are independent of the first's sums (1.1 of the
+    thermodynamics' time where loads of several species are in flight, 1.35 with one at a time)."""
+    mech = synth.mechanism("ch4_53sp_325rx")
+    m = gpu_mechanism("ch4_53sp_325rx")
+    n = 5000
+    st = synth.states_uniform(mech.K, n, seed=2)
+    T, p, Y = to_dev(st.T, st.p, st.Y)
+    D, G = torch.rand_like(Y), torch.randn((3, mech.K, n), dtype=torch.float64, device="cuda")
+    many = lambda f: _median_ms(lambda: [f() for _ in range(20)])                             # noqa: E731
+    flux, thermo = many(lambda: nk.diffusion_fluxes(m, T, p, Y, D, G)), many(lambda: nk.thermo_eval(m, T, p, Y))
+    assert flux <= 1.15 * thermo, (flux, thermo)
