@@ -549,6 +549,27 @@ cudaError_t launch_marked(const DevMech& m, int64_t n, int64_t ld, const double*
 
 int64_t linc_slots(const DevMech& m) { return cs_C(m) + m.K; }
 
+namespace {
+// Few species: the pair kernel runs one thread a point, which keeps twice the points resident that the chunked
+// kernel does, and its wave costs 1.75 of the chunked one's (9 species / 21 reactions: 39.4 us for up to 58,368
+// points against 23.6 for 29,184; by counts of waves 1 : 2 old 39.4, new 46.7 us; 2 : 3 84.6 and 72.0; 5 : 9
+// 210 and 229; 18 : 35 724 and 823).  The sources' products, whose epilogue all parts share in the chunked kernel,
+// break even at 1.9 up to 16 species and lose nothing above; the rates' need 2 waves to one above 24 species
+// (28 species / 110 reactions, 40,000 points, 1 : 2: 191 and 210) and break even at 32.
+bool jvpc_pair_wins(const DevMech& m, int64_t n, int rhs) {
+    if (m.K > (rhs ? 16 : 31) || n <= 16384) return false;      // (fewer points than one wave of either)
+    const int idx = rhs ? plan_shape<3>(m.K) : plan_shape<2>(m.K);
+    if (idx < 0 || kShapes[idx].np != 1) return false;
+    const auto seq = std::make_integer_sequence<int, kNumShapes>{};
+    const int64_t w = wave_points(rhs ? kernel_ptr<3>(idx, seq) : kernel_ptr<2>(idx, seq), kShapes[idx].blk,
+                                  mode_smem(m.K, kShapes[idx], rhs ? 3 : 2), kShapes[idx].blk);
+    const int64_t v = wave_points(rhs ? (const void*)jvpc_fx_kernel<4, true> : (const void*)jvpc_fx_kernel<4, false>, 128,
+                                  jvpc_fx_smem(m), 32);
+    if (w == 0 || v == 0) return false;
+    return 100 * ((n + v - 1) / v) >= (rhs ? 190 : m.K > 24 ? 200 : 180) * ((n + w - 1) / w);
+}
+}  // namespace
+
 cudaError_t launch_linearize_compact(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                                      const double* Y, const double* dlnA, double* lin, int64_t ldl, double* omega,
                                      double* hrr, cudaStream_t s) {
@@ -577,7 +598,7 @@ cudaError_t launch_jvp_linearized_compact(const DevMech& m, int64_t n, int64_t l
                                           const double* Y, const double* lin, int64_t ldl, const double* fT,
                                           const double* fY, int64_t ldf, const double* vT, const double* vY,
                                           double* d_T, double* d_Y, cudaStream_t s, int rhs) {
-    if (m.fx_ok && m.K >= 3 && jvpc_fx_smem(m) <= smem_limit())
+    if (m.fx_ok && m.K >= 3 && jvpc_fx_smem(m) <= smem_limit() && !jvpc_pair_wins(m, n, rhs))
         return rhs ? launch_jvpc_fx<true>(m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, fT, fY, ldf, s)
                    : launch_jvpc_fx<false>(m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, nullptr, nullptr, 0, s);
     if (rhs) {

@@ -140,6 +140,30 @@ cudaError_t ensure_smem(const void* kernel, size_t bytes) {
     return cudaSuccess;
 }
 
+namespace {
+struct WaveEntry {
+    const void* kernel;
+    int device, threads;
+    size_t smem;
+    int64_t blocks;
+};
+std::mutex g_wave_mu;
+std::vector<WaveEntry> g_wave;
+}  // namespace
+
+int64_t wave_points(const void* kernel, int threads, size_t smem, int points) {
+    int dev = 0, sms = 0, per_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || ensure_smem(kernel, smem) != cudaSuccess) return 0;
+    std::lock_guard<std::mutex> lk(g_wave_mu);
+    for (const WaveEntry& w : g_wave)
+        if (w.kernel == kernel && w.device == dev && w.threads == threads && w.smem == smem) return w.blocks * points;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess)
+        return 0;
+    if (g_wave.size() < 256) g_wave.push_back({kernel, dev, threads, smem, (int64_t)sms * per_sm});
+    return (int64_t)sms * per_sm * points;
+}
+
 size_t smem_limit() {
     int dev = 0, v = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 48 * 1024;

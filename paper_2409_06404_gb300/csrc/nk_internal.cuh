@@ -447,6 +447,9 @@ int pick_block(size_t bytes_per_thread, size_t budget);
 int pick_block_occupancy(size_t bytes_per_thread, size_t fixed_bytes, size_t bytes_per_warp = 0);
 // Opt a kernel into `bytes` of dynamic shared memory on the current device (cached).
 cudaError_t ensure_smem(const void* kernel, size_t bytes);
+// Points that a kernel has resident on the whole device at once (occupancy x SMs x points of a block; cached),
+// 0 if it cannot be told.
+int64_t wave_points(const void* kernel, int threads, size_t smem, int points);
 // Opt-in shared-memory limit per block of the current device.
 size_t smem_limit();
 

@@ -179,3 +179,33 @@ def test_fluxes_of_few_points(cuda):
     many = lambda f: _median_ms(lambda: [f() for _ in range(20)])                             # noqa: E731
     flux, thermo = many(lambda: nk.diffusion_fluxes(m, T, p, Y, D, G)), many(lambda: nk.thermo_eval(m, T, p, Y))
     assert flux <= 1.15 * thermo, (flux, thermo)
+
+
+@pytest.mark.parametrize("K,R,n", [(9, 21, 29184), (9, 21, 45000), (9, 21, 90000), (16, 48, 45000), (24, 60, 45000)])
+def test_products_of_few_species(cuda, K, R, n):
+    """Products from stored data at few species, where the number of points chooses between the chunked and
+    the pair kernel: the compact ones against the oracle at 200 points, the single-precision ones bit
+    for bit against blocks of 1,000 points, which the chunked kernel takes."""
+    el = ("H", "O", "N") if K < 20 else ("C", "H", "O", "N")
+    mech = synth.make_mechanism(K, R, 2, 2, elements=el, seed=900 + K)
+    m = gpu_mechanism(mech)
+    st = synth.states_uniform(K, n, seed=K)
+    vT, vY = synth.normal(n, 1), synth.normal((K, n), 2)
+    S, (vTt, vYt) = to_dev(st.T, st.p, st.Y), to_dev(vT, vY)
+    fT, fY = nk.rhs_eval(m, *S)
+    lin = nk.rates_linearize_compact(m, *S)
+    i = np.sort(np.random.default_rng(3).choice(n, 200, replace=False))
+    sub = lambda a: np.ascontiguousarray(a[..., i])                                           # noqa: E731
+    for got, ref in ((nk.rates_jvp_linearized_compact(m, *S, lin, vTt, vYt), oracle.jvp),
+                     (nk.rhs_jvp_linearized_compact(m, *S, lin, fT, fY, vTt, vYt), oracle.rhs_jvp)):
+        want = ref(mech, sub(st.T), sub(st.p), sub(st.Y), sub(vT), sub(vY), scales=True)
+        for a, o, s in zip(got, want[:2], want[2:]):
+            assert scaled_err(sub(host(a)), o, s) <= TOL
+    lin = nk.rates_linearize_f32(m, *S)
+    whole = nk.rates_jvp_linearized_f32(m, *S, lin, vTt, vYt) + nk.rhs_jvp_linearized_f32(m, *S, lin, fT, fY, vTt, vYt)
+    for a in range(0, n, 10000):
+        b = min(a + 1000, n)
+        x = [t[..., a:b].contiguous() for t in (*S, lin, fT, fY, vTt, vYt)]
+        part = nk.rates_jvp_linearized_f32(m, *x[:4], *x[6:]) + nk.rhs_jvp_linearized_f32(m, *x)
+        assert all(torch.equal(q, w[..., a:b]) for q, w in zip(part, whole))
+    m.close()
