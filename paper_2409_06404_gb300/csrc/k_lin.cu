@@ -885,6 +885,23 @@ cudaError_t launch_linearize_f32(const DevMech& m, int64_t n, int64_t ld, const 
                          lin, ldl);
 }
 
+namespace {
+// The pair kernel's shape of one thread a point keeps three times the points of the chunked kernel resident and has
+// no barriers: with fewer than a dozen species and three reactions a species or fewer it is the better one where
+// the chunked kernel needs 2.75 waves or more for each of its (9 species / 21 reactions, sources' product: 90,000
+// points, 1 : 3 waves, 45.6 and 57.5 us; 1,000,000 points, 9 : 26, 529 and 613; 262,144 points, 3 : 7, 173 and 162).
+bool lin32_pair_wins(const DevMech& m, int64_t n, int idx, bool rhs) {
+    if (m.K >= 12 || m.R > 3 * m.K || kShapes[idx].np != 1 || n <= 16384) return false;
+    const auto seq = std::make_integer_sequence<int, kNumShapes>{};
+    const int64_t w = wave_points(rhs ? kernel_ptr<4>(idx, seq) : kernel_ptr<3>(idx, seq), kShapes[idx].blk,
+                                  lin_smem(m.K, kShapes[idx], rhs ? 4 : 3), kShapes[idx].blk);
+    const int64_t v = wave_points(rhs ? (const void*)jvp_lin32_fx_kernel<4, 1, true> : (const void*)jvp_lin32_fx_kernel<4, 1, false>,
+                                  128, lin32_fx_smem(lin32_set(m, 1), m.K, 1), 32);
+    if (w == 0 || v == 0) return false;
+    return 4 * ((n + v - 1) / v) >= 11 * ((n + w - 1) / w);
+}
+}  // namespace
+
 cudaError_t launch_jvp_linearized_f32(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                                       const double* Y, const float* lin, int64_t ldl, const double* fT,
                                       const double* fY, int64_t ldf, const double* vT, const double* vY,
@@ -892,14 +909,14 @@ cudaError_t launch_jvp_linearized_f32(const DevMech& m, int64_t n, int64_t ld, c
     if (rhs) {
         const int idx = plan_shape<4>(m.K);
         if (idx < 0) return cudaErrorInvalidConfiguration;
-        if (lin32_fx_fits(m, kShapes[idx].np))
+        if (lin32_fx_fits(m, kShapes[idx].np) && !lin32_pair_wins(m, n, idx, true))
             return launch_lin32_fx<true>(kShapes[idx].np, m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, fT, fY, ldf, s);
         return launch_idx<4>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, lin,
                              ldl, vT, vY, d_Y, d_T, fT, fY, ldf);
     }
     const int idx = plan_shape<3>(m.K);
     if (idx < 0) return cudaErrorInvalidConfiguration;
-    if (lin32_fx_fits(m, kShapes[idx].np))
+    if (lin32_fx_fits(m, kShapes[idx].np) && !lin32_pair_wins(m, n, idx, false))
         return launch_lin32_fx<false>(kShapes[idx].np, m, n, ld, T, p, Y, lin, ldl, vT, vY, d_Y, d_T, nullptr, nullptr, 0, s);
     const double* none = nullptr;
     return launch_idx<3>(idx, std::make_integer_sequence<int, kNumShapes>{}, m.K, n, s, m, n, ld, T, p, Y, lin, ldl,

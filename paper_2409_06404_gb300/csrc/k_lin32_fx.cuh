@@ -174,18 +174,36 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
         if (part + NP * j < K) sW[__ldg(&f.sp[part + NP * j].k) * 32] = w[j];
     __syncthreads();
 
-    // the epilogue of jvp_lin32_kernel by its number of parts
-    if (part >= OLD) return;
+    // The epilogue of jvp_lin32_kernel: the outputs by all parts, which leave what the point sums take in
+    // shared memory (h_k/RT in the rows of dC_k, the sources' y_k and v_k in the reactions' rows where they
+    // fit); the sums by the old number of parts.  (All of it by one part of four: 9 species / 21
+    // reactions, 1,000,000 points, sources' product 763 us instead of 613.)
     const double Td = T[i], dTd = vT[i];
     const float Ti = narrow(Td), dT = narrow(dTd), rho = sV[32], arho = sV[64];
-    double hsum = 0.0;
-    float cpm = 0.0f, dcpm = 0.0f;
     const float inv_rho = RHS ? 1.0f / rho : 0.0f;
     const double arho_d = widen(arho);
+    float* sH = reinterpret_cast<float*>(sdC);
+    const bool stash = RHS && K <= f.rows;
+#pragma unroll 2
+    for (int k = part; k < K; k += NP) {
+        double dw = scale2(widen(sW[k * 32]), sE[k * 32]);
+        sH[k * 32] = lin[(slot_H32(m) + k) * ldl + i];
+        if constexpr (RHS) {
+            const float iw = __ldg(m.f_invW + k);
+            if (stash)
+                *reinterpret_cast<float2*>(sQ + k * 256) =
+                    make_float2(narrow(Y[(int64_t)k * ld + i]) * iw, narrow(vY[(int64_t)k * ld + i]) * iw);
+            dw = fma(widen(inv_rho / iw), dw, -fY[(int64_t)k * ldf + i] * arho_d);
+        }
+        if (live) d_omega[(int64_t)k * ld + i] = dw;
+    }
+    __syncthreads();
+    if (part >= OLD) return;
+    double hsum = 0.0;
+    float cpm = 0.0f, dcpm = 0.0f;
 #pragma unroll 2
     for (int k = part; k < K; k += OLD) {
-        double dw = scale2(widen(sW[k * 32]), sE[k * 32]);
-        hsum = fma(widen(lin[(slot_H32(m) + k) * ldl + i]), dw, hsum);
+        hsum = fma(widen(sH[k * 32]), scale2(widen(sW[k * 32]), sE[k * 32]), hsum);
         if constexpr (RHS) {
             const bool lo = __double_as_longlong(Td) <= __ldg(reinterpret_cast<const long long*>(m.Tmid) + k);
             const float* cf = m.f_cp + ((size_t)k * 2 + (lo ? 0 : 1)) * 8;
@@ -193,13 +211,16 @@ __global__ void __launch_bounds__(32 * NP, NP == 4 ? 8 : NP == 8 ? 4 : NP == 16 
             const float a5 = __ldg(cf + 4);
             const float cpk = fmaf(Ti, fmaf(Ti, fmaf(Ti, fmaf(Ti, a5, c.w), c.z), c.y), c.x);
             const float dcpk = fmaf(Ti, fmaf(Ti, fmaf(Ti, 4.0f * a5, 3.0f * c.w), 2.0f * c.z), c.y);
-            const float iw = __ldg(m.f_invW + k);
-            const float yk = narrow(Y[(int64_t)k * ld + i]) * iw, vk = narrow(vY[(int64_t)k * ld + i]) * iw;
-            cpm = fmaf(yk, cpk, cpm);
-            dcpm = fmaf(vk, cpk, fmaf(yk * dcpk, dT, dcpm));
-            dw = fma(widen(inv_rho / iw), dw, -fY[(int64_t)k * ldf + i] * arho_d);
+            float2 yv;
+            if (stash) {
+                yv = *reinterpret_cast<const float2*>(sQ + k * 256);
+            } else {
+                const float iw = __ldg(m.f_invW + k);
+                yv = make_float2(narrow(Y[(int64_t)k * ld + i]) * iw, narrow(vY[(int64_t)k * ld + i]) * iw);
+            }
+            cpm = fmaf(yv.x, cpk, cpm);
+            dcpm = fmaf(yv.y, cpk, fmaf(yv.x * dcpk, dT, dcpm));
         }
-        if (live) d_omega[(int64_t)k * ld + i] = dw;
     }
     if constexpr (OLD > 1) {
         sR[part * 32] = hsum;
