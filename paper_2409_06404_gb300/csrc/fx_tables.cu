@@ -305,6 +305,7 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
                 for (int j = 0; j < 18; ++j) {
                     long double& m = most[j < 5 ? 0 : j < 11 ? 1 : 2];
                     m = std::max(m, fabsl(c[r][j]));
+                    th = th && std::isfinite((double)c[r][j]);      // (a NaN or infinite coefficient: doubles)
                 }
             }
             for (int q = 0; q < 3; ++q) {
@@ -366,8 +367,10 @@ FxTables build_fx_tables(int K, const std::vector<RxnRec>& rxn, const std::vecto
     }
     // (eps - 1)/W relative to the largest 1/W, in units of 2^(eff_shift - 62)
     long double m = 1.0L;
-    for (size_t j = 0; j < eff_sp.size(); ++j)
+    for (size_t j = 0; j < eff_sp.size(); ++j) {
         m = std::max(m, fabsl((long double)eff_m1[j]) / (long double)W[eff_sp[j]] / maxInv);
+        ok = ok && std::isfinite(eff_m1[j]);                        // (std::max passes a NaN over)
+    }
     while (ldexpl(1.0L, f.eff_shift) <= m && f.eff_shift < 32) ++f.eff_shift;
     if (f.eff_shift >= 20) ok = false;
     std::vector<double> eff_w(eff_sp.size());

@@ -209,3 +209,31 @@ def test_products_of_few_species(cuda, K, R, n):
         part = nk.rates_jvp_linearized_f32(m, *x[:4], *x[6:]) + nk.rhs_jvp_linearized_f32(m, *x)
         assert all(torch.equal(q, w[..., a:b]) for q, w in zip(part, whole))
     m.close()
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_nonfinite_mechanism_constants(cuda, bad):
+    """A NaN or infinite polynomial coefficient, or efficiency of a falloff reaction, reaches what depends on
+    it, as in the oracle, and nothing else."""
+    base = synth.mechanism("h2_9sp_21rx")
+    st = synth.states_uniform(base.K, 64, seed=6)
+    T = np.linspace(400.0, 2200.0, 64)
+    S = to_dev(T, st.p, st.Y)
+    mech = base.copy()
+    mech.nasa_hi[3, 2] = bad
+    m = gpu_mechanism(mech)
+    got, want = nk.thermo_eval(m, *S), oracle.thermo(mech, T, st.p, st.Y)
+    for key in ("cp_k", "h_k", "g_k", "cp_mix", "h_mix"):
+        a, o = host(got[key]), np.asarray(want[key])
+        assert np.array_equal(np.isfinite(a), np.isfinite(o)), key
+        ok = np.isfinite(o)
+        assert np.allclose(a[ok], o[ok], rtol=1e-11), key
+    m.close()
+    mech = base.copy()
+    r = int(np.flatnonzero(mech.rtype == 2)[0])
+    mech.eff[r, 2] = bad
+    m = gpu_mechanism(mech)
+    w = host(nk.rates_eval(m, *S)[0])
+    wo = oracle.rates(mech, T, st.p, st.Y)[0]
+    assert np.array_equal(np.isfinite(w), np.isfinite(wo))
+    m.close()
