@@ -2,6 +2,8 @@
 cancel, fields with points outside the form in some or all blocks.
 
 Tolerance 1e-10 of the cancellation-aware scales, as for every derivative kernel here."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -236,4 +238,31 @@ def test_nonfinite_mechanism_constants(cuda, bad):
     w = host(nk.rates_eval(m, *S)[0])
     wo = oracle.rates(mech, T, st.p, st.Y)[0]
     assert np.array_equal(np.isfinite(w), np.isfinite(wo))
+    m.close()
+
+
+@pytest.mark.parametrize("K,R,n", [(9, 20, 33), (9, 48, 1), (32, 49, 64), (33, 36, 97), (53, 325, 160), (65, 97, 96), (140, 150, 65)])
+def test_solver_linearization(cuda, K, R, n):
+    """The per-entry linearization that the reactor keeps to itself (fixed-point pass, pair kernel for blocks
+    outside its form: the second block here): products from it against the oracle."""
+    el = ("H", "O", "N") if K < 20 else ("C", "H", "O", "N")
+    mech = synth.make_mechanism(K, R, max(1, R // 16), max(1, R // 13), elements=el, seed=650 + K)
+    m = gpu_mechanism(mech)
+    st = synth.states_uniform(K, n, seed=K)
+    T, Y = st.T.copy(), st.Y.copy()
+    if n >= 64:
+        T[33] = 4500.0
+        Y[2, 34], Y[K - 1, 35] = 0.0, -1e-4
+    if n >= 96:
+        Y[K - 1, 70] = -1e-4
+    vT, vY, dA = synth.normal(n, 1), synth.normal((K, n), 2), 0.1 * synth.normal(R, 3)
+    S, (vTt, vYt, dAt) = to_dev(T, st.p, Y), to_dev(vT, vY, dA)
+    lin = torch.empty((nk.linearization_slots(m), n), dtype=torch.float64, device="cuda")
+    f = nk.lib()["_ZN2nk23launch_linearize_solverERKNS_7DevMechEllPKdS4_S4_S4_PdlP11CUstream_st"]
+    f.argtypes = [ctypes.c_void_p] + [ctypes.c_int64] * 2 + [ctypes.c_void_p] * 5 + [ctypes.c_int64, ctypes.c_void_p]
+    P = lambda t: t.data_ptr()                                                                # noqa: E731
+    assert f(m.handle, n, n, *map(P, S), P(dAt), P(lin), n, torch.cuda.current_stream().cuda_stream) == 0
+    a, b = nk.rates_jvp_linearized(m, *S, lin, vTt, vYt)
+    dw, dh, dws, dhs = oracle.jvp(mech, T, st.p, Y, vT, vY, dlnA=dA, scales=True)
+    assert scaled_err(host(a), dw, dws) <= TOL and scaled_err(host(b), dh, dhs) <= TOL
     m.close()
