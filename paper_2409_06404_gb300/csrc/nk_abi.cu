@@ -540,26 +540,6 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
             for (int j = 0; j < 5; ++j)
                 f_cp[((size_t)k * 2 + range) * 8 + j] = (float)nasa[((size_t)k * 2 + range) * nk::kNasaStride + j];
 
-    // log2(1/D_jk) at p_ref as a cubic in log2(T)/32, 64-bit integers in units of 2^-48 (+2: fx_mul cuts),
-    // where every coefficient and, over 128..4096 K, every value stays in range
-    std::vector<int64_t> tr_D((size_t)P * 4 + 4, 0);
-    bool tr_ok = true;
-    {
-        const double l2e = 1.4426950408889634074, ln2 = 0.69314718055994530942;
-        for (int q = 0; q < P && tr_ok; ++q) {
-            const double* a = d->D_fit + 4 * (size_t)q;
-            long double b = 1.0L;
-            for (int j = 0; j < 4; ++j, b *= 0.693147180559945309417232121458L * 32.0L) {
-                const long double c = -1.44269504088896340735992468100189214L * a[j] * b;
-                tr_ok = tr_ok && fabsl(c) < 15000.0L;
-                tr_D[4 * (size_t)q + j] = tr_ok ? (int64_t)llroundl(c * 281474976710656.0L) + (j == 0 ? 2 : 0) : 0;
-            }
-            for (int t = 0; t <= 16 && tr_ok; ++t) {
-                const double lnT = ln2 * (7.0 + 5.0 * t / 16.0);
-                tr_ok = std::fabs(l2e * (a[0] + lnT * (a[1] + lnT * (a[2] + lnT * a[3])))) < 60.0;
-            }
-        }
-    }
     std::vector<int> order32[3];
     for (int q = 0; q < R; ++q) order32[0].push_back(q);
     for (int v = 0; v < 2; ++v)
@@ -597,7 +577,7 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
                  o_xr = L.add(fxt.set[0].chunks.size() + 16), o_xr1 = L.add(fxt.set[1].chunks.size() + 16),
                  o_xr2 = L.add(fxt.set[2].chunks.size() + 16), o_xn = L.add((size_t)R * 4 + 16),
                  o_y0 = L.add(fxt.set32[0].chunks.size() + 16), o_y1 = L.add(fxt.set32[1].chunks.size() + 16),
-                 o_y2 = L.add(fxt.set32[2].chunks.size() + 16), o_trD = L.add(tr_D.size() * 8), o_ys = L.add((size_t)K * 4 + 16),
+                 o_y2 = L.add(fxt.set32[2].chunks.size() + 16), o_ys = L.add((size_t)K * 4 + 16),
                  o_xs2 = L.add(fxt.set[2].sp.size() * sizeof(nk::FxSpecies) + 16),
                  o_xx = L.add(fxt.extra.size() * sizeof(nk::FxExtra) + 16),
                  o_xt = L.add(fxt.troe.size() * sizeof(nk::FxTroe) + 16),
@@ -673,7 +653,6 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
     put(o_y0, fxt.set32[0].chunks.data(), fxt.set32[0].chunks.size());
     put(o_y1, fxt.set32[1].chunks.data(), fxt.set32[1].chunks.size());
     put(o_y2, fxt.set32[2].chunks.data(), fxt.set32[2].chunks.size());
-    put(o_trD, tr_D.data(), tr_D.size() * 8);
     put(o_ys, fxt.slot32.data(), fxt.slot32.size() * 4);
     put(o_xn, fxt.nu1.data(), fxt.nu1.size() * 4);
     put(o_xs1, fxt.set[1].sp.data(), fxt.set[1].sp.size() * sizeof(nk::FxSpecies));
@@ -771,8 +750,6 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
     dm.mt_eps4 = reinterpret_cast<const double*>(b + o_me4);
     dm.fx_ok = fxt.ok ? 1 : 0;
     dm.th_lo = fxt.th_lo;
-    dm.tr_ok = tr_ok ? 1 : 0;
-    dm.tr_D = reinterpret_cast<const int64_t*>(b + o_trD);
     dm.th = reinterpret_cast<const nk::FxThermo*>(b + o_th);
     dm.fxs[0] = fxt.set[0].s;
     dm.fxs[0].chunks = b + o_xr;
@@ -792,7 +769,6 @@ nk_status nk_mechanism_load(const nk_mech_desc* d, nk_mech** out) {
     dm.fxs[1].sp = reinterpret_cast<const nk::FxSpecies*>(b + o_xs1);
     dm.fx_eff_shift = fxt.eff_shift;
     dm.fx_lmaxw = (int64_t)llroundl((long double)fxt.log2_maxinvW * 281474976710656.0L);
-    dm.fx_maxw = *std::max_element(invW.begin(), invW.end());
     dm.fx_lR = (int64_t)llroundl(log2l((long double)nk::kR) * 281474976710656.0L);
     dm.fx_tab = reinterpret_cast<const uint32_t*>(b + o_xtab);
     dm.fx_extra = reinterpret_cast<const nk::FxExtra*>(b + o_xx);

@@ -151,38 +151,6 @@ __device__ __forceinline__ double fx_exp2(long long x, const FxTab& t) {
     return __hiloint2double((int)hi, (int)lo32);
 }
 
-// 2^x as a pair, for |x| < 100: fx_exp2's steps up to T_j (1 + (2^r' - 1)), then 2^m on both halves
-__device__ __forceinline__ dfl fx_exp2_pair(long long x, const uint2* tab) {
-    const int xh = (int)(x >> 32);
-    const uint2 en = tab[(xh >> 9) & 127];
-    const unsigned long long R = (((unsigned long long)((uint32_t)xh & 0x1ffu) << 32) | (uint32_t)x) + en.y;
-    const float fh = __fsub_rn(__int_as_float(0x4B000000 | (int)(R >> 19)), 8388608.0f);
-    const float fl = __fsub_rn(__int_as_float(0x4B000000 | (int)((uint32_t)R & 0x7ffffu)), 8388608.0f);
-    constexpr float c1 = 0.693147182464599609375f * 0x1p-29f, c2 = -1.9046542121259336e-09f * 0x1p-29f;
-    constexpr float c3 = 0.693147182464599609375f * 0x1p-48f;
-    const float p = __fmul_rn(fh, c1);
-    float e = __fmaf_rn(fh, c1, -p);
-    e = __fmaf_rn(fh, c2, e);
-    e = __fmaf_rn(fl, c3, e);
-    const float q = __fmul_rn(p, p);
-    const float qe = __fmaf_rn(p, p, -q);
-    const float s = __fmaf_rn(0.5f, q, p);
-    float lo = __fmaf_rn(0.5f, q, -__fsub_rn(s, p));
-    const float tl = __fmaf_rn(p, __fmaf_rn(p, 1.0f / 120.0f, 1.0f / 24.0f), 1.0f / 6.0f);
-    float w = __fmaf_rn(__fmul_rn(q, p), tl, e);
-    w = __fmaf_rn(0.5f, qe, w);
-    w = __fmaf_rn(s, e, w);
-    lo = __fadd_rn(lo, w);
-    const float T = __uint_as_float(en.x);
-    const float v = __fmul_rn(T, s);
-    float ve = __fmaf_rn(T, s, -v);
-    ve = __fmaf_rn(T, lo, ve);
-    const float h = __fadd_rn(T, v);
-    const float l = __fadd_rn(__fsub_rn(v, __fsub_rn(h, T)), ve);
-    const float sc = __int_as_float((127 + (xh >> 16)) << 23);
-    return {__fmul_rn(h, sc), __fmul_rn(l, sc)};
-}
-
 // x 2^-48 as a double, by integer operations
 __device__ __forceinline__ double fx_to_d(long long x) {
     const unsigned long long a = (unsigned long long)(x < 0 ? -x : x);

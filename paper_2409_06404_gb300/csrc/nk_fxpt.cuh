@@ -4,7 +4,7 @@
 // A block takes 32 points, one lane each, and NP warps ("parts") share a point.  Species k belongs
 // to part k % NP (at most kFxOwn species per part); the parts take the reactions of a chunk in
 // turn and leave their rates of progress in shared memory, and each part then sums its own
-// species over the chunk's list (FxTables): two barriers per chunk of 64 reactions, where adding
+// species over the chunk's list (FxTables): two barriers per chunk of up to 48 reactions, where adding
 // into the species' rows directly took one per round of reactions without a common species (84
 // rounds at 325 reactions), and no reaction waits for another.  The order of every sum is fixed by
 // the mechanism.

@@ -112,7 +112,8 @@ static_assert(sizeof(FxRxn) == 64, "fixed-point reaction record");
 struct __align__(16) FxExtra {
     int32_t eff0, eff1, aux, pad;  // third-body efficiencies [eff0, eff1), Troe record or -1
 };
-// Chunks: up to FxSet::chunk reactions whose rates of progress are staged together.  A chunk's image
+// Chunks: up to 48 reactions (36 in the derivative kernels of up to 12 parts; fx_tables.cu) whose rates of
+// progress are staged together.  A chunk's image
 // (fx_image bytes, a multiple of 16) holds its reaction records in schedule order (part by part,
 // balanced by cost), then at image_parts the first record of each part (NP + 1 bytes), at
 // image_spec one word per species slot (start in the list << 16 | rows to add << 8 | rows to
@@ -284,7 +285,6 @@ struct DevMech {
     FxSet fx32[3];                // the single-precision products, summed as by 1, 2, 4 parts' rounds
     const int32_t* fx32_slot;     // [K] slot of a species in them
     int64_t fx_lmaxw, fx_lR;      // log2(largest 1/W), log2(R)
-    double fx_maxw;               // largest 1/W
     const uint32_t* fx_tab;
     const FxExtra* fx_extra;
     const int32_t* fx_nu1;        // [R] first reactant's coefficient | first product's << 4 (device order)
@@ -292,8 +292,6 @@ struct DevMech {
     const FxEff* fx_eff;
     // fixed-point thermo polynomials (th_lo: low-range fraction T/2^th_lo; 0: they do not fit)
     int32_t th_lo;
-    int32_t tr_ok;                // the binary diffusion fits in fixed point (128 < T < 4096 K)
-    const int64_t* tr_D;          // [P][4] -log2 D_jk: cubic in log2(T)/32 (fx_mul's halving included)
     const FxThermo* th;
 };
 
