@@ -7,7 +7,7 @@
 // 4.2 cycles per issue, issue slots 51% busy), so a reaction's words are loaded while the one before
 // is summed, and all parts load the state.  53 species, 2,097,152 points: 12.6 -> 9.0 ms per product
 // (2.3 TB/s of the stored words); the single-precision stage of 175,616 points with its ten
-// products: 21.7 -> 15.8 ms.
+// products: 21.7 -> 15.7 ms.
 #pragma once
 
 #include "nk_fxpt.cuh"

@@ -2,8 +2,10 @@
 // included by k_lin.cu, whose slots and store_coef it uses): an entry's coefficient is its side's term
 // divided by the concentration, nu_e q_side / C_e, one product with a row of 1/C_k, where the pair
 // kernel formed exclusive products of the concentrations.  The stored words bound it together with
-// the FP64 pipe (one quotient's product per entry).  Block-Jacobi set-up and reactor steps, which
-// read the stored entries, 53 species, 16,384 points: 9.50 -> 8.87 ms.
+// the FP64 pipe (one quotient's product per entry).  53 species, states in the form: 16,384 points 0.42 ms by
+// the pair kernel in four parts a point -> 0.245, 262,144 points 6.04 -> 3.10.  (Near-equilibrium states, whose
+// rare species lie below 2^-100, stay with the pair kernel; a reactor step on 16,384 of them went from 9.50 to
+// 8.44 ms by its launch shape, k_lin.cu, and by what the factorization gained.)
 // For linearizations a solver keeps to itself; the public one and the single-precision data rounded
 // from it stay with the pair kernel: two linearizations that differ by 3e-13 round some hundred
 // coefficients of a field to the other float, 6e-8 of a product.
