@@ -658,12 +658,13 @@ const void* kernel_ptr(int c) {
 // Per pass: the parts per point with the most resident warps and a grid of resident blocks (the
 // fallback pass finds work only in tiles with mass fractions or cotangents outside the pairs'
 // range; it reads the rest's Y and bar_omega once to see that).  The ln A partial sums of the two
-// passes' blocks lie one after the other in the workspace (behind the fixed-point kernel: vjp_rows_used).
+// passes' blocks lie one after the other in the workspace (behind the fixed-point kernel they add to its rows).
 struct VjpPlan {
     int dev, K, R, ms2, ms4, variant;
     int parts_idx[2];   // index into kParts, per pass
     int grid_cap[2];    // blocks of each pass
     int fx_cap;         // blocks of the fixed-point kernel (0: it does not take the mechanism)
+    int sms;
 };
 std::mutex g_plan_mu;
 std::vector<VjpPlan> g_plans;
@@ -712,7 +713,7 @@ bool plan_variant(const DevMech& m, VjpPlan& out) {
     int p0 = -1, p1 = -1, b0 = 0, b1 = 0;
     if (!plan_pass<WANT_G, HB, 0>(m, sms, per_block, p0, b0)) return false;
     if (!plan_pass<WANT_G, HB, 1>(m, sms, per_block, p1, b1)) return false;
-    out = VjpPlan{dev, m.K, m.R, m.mslots2, m.mslots4, variant, {p0, p1}, {sms * b0, sms * b1}, 0};
+    out = VjpPlan{dev, m.K, m.R, m.mslots2, m.mslots4, variant, {p0, p1}, {sms * b0, sms * b1}, 0, sms};
     if (vjp_fx_fits(m)) out.fx_cap = sms * std::min(vjp_fx_blocks(m), b0 + b1);
     std::lock_guard<std::mutex> lk(g_plan_mu);
     g_plans.push_back(out);
@@ -737,22 +738,25 @@ int64_t vjp_fx_grid(const VjpPlan& pl, int64_t n) {
 // The ln A partial sums' rows in the workspace: one per block of the two passes.
 int64_t vjp_rows(const VjpPlan& pl, int64_t n) { return vjp_grid(pl, 0, n) + vjp_grid(pl, 1, n); }
 
-// The rows that a call writes.  Behind the fixed-point kernel the passes add to its rows, so that the
-// workspace needs no more rows than the two passes alone (fx_cap is at most the sum of their caps).
-int64_t vjp_rows_used(const VjpPlan& pl, int64_t n) {
-    return pl.fx_cap ? std::max({vjp_fx_grid(pl, n), vjp_grid(pl, 0, n), vjp_grid(pl, 1, n)}) : vjp_rows(pl, n);
+// The least rows a call does with.  Behind the fixed-point kernel the passes add to its rows, so fewer rows only
+// mean fewer blocks: that kernel's and half a block per SM for each pass.
+int64_t vjp_rows_least(const VjpPlan& pl, int64_t n) {
+    const int64_t rows = vjp_rows(pl, n), tiles = (n + kVjpBlk - 1) / kVjpBlk;
+    if (!pl.fx_cap) return rows;
+    const int64_t caps = pl.grid_cap[0] + pl.grid_cap[1], fx = std::min<int64_t>(pl.fx_cap, std::max<int64_t>(pl.sms, caps - pl.sms));
+    return std::min(rows, std::min(tiles, fx) + 2 * std::min<int64_t>(tiles, std::max(1, pl.sms / 2)));
 }
 
 template <bool WANT_G, bool HB, int PASS, bool MARKED = false>
 cudaError_t launch_pass(const VjpPlan& pl, const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                         const double* Y, const double* dlnA, const double* bar_omega, const double* bar_hrr,
-                        double* gT, double* gY, double* ws, int64_t have, cudaStream_t s) {
+                        double* gT, double* gY, double* ws, int64_t blocks, int64_t have, cudaStream_t s) {
     const int np = kParts[pl.parts_idx[PASS]];
     const size_t smem = vjp_smem(m.K, m.R, vjp_mslots(m, np), WANT_G);
     const void* kp = kernel_ptr<WANT_G, HB, PASS, MARKED>(pl.parts_idx[PASS]);
     cudaError_t e = ensure_smem(kp, smem);
     if (e != cudaSuccess) return e;
-    const unsigned grid = (unsigned)vjp_grid(pl, PASS, n);
+    const unsigned grid = (unsigned)blocks;
     switch (np) {
         case 1:
             vjp_kernel<1, WANT_G, HB, PASS, MARKED><<<grid, kVjpBlk, smem, s>>>(m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr,
@@ -769,23 +773,27 @@ cudaError_t launch_pass(const VjpPlan& pl, const DevMech& m, int64_t n, int64_t 
     return cudaGetLastError();
 }
 
+// max_rows: rows of the workspace; used: the rows written.
 template <bool WANT_G, bool HB>
 cudaError_t launch_v(const VjpPlan& pl, const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                      const double* Y, const double* dlnA, const double* bar_omega, const double* bar_hrr, double* gT,
-                     double* gY, double* ws, cudaStream_t s) {
+                     double* gY, double* ws, int64_t max_rows, int64_t& used, cudaStream_t s) {
+    const int64_t g0 = vjp_grid(pl, 0, n), g1 = vjp_grid(pl, 1, n);
     if (pl.fx_cap) {
-        const int64_t g = vjp_fx_grid(pl, n), g0 = vjp_grid(pl, 0, n);
+        const int64_t g = std::min(vjp_fx_grid(pl, n), max_rows), h0 = std::min(g0, max_rows), h1 = std::min(g1, max_rows);
+        used = std::max({g, h0, h1});
         cudaError_t e = launch_vjp_fx<WANT_G, HB>(m, g, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, s);
         if (e != cudaSuccess) return e;
-        e = launch_pass<WANT_G, HB, 0, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, g, s);
+        e = launch_pass<WANT_G, HB, 0, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, h0, g, s);
         if (e != cudaSuccess) return e;
-        return launch_pass<WANT_G, HB, 1, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws,
-                                                std::max(g, g0), s);
+        return launch_pass<WANT_G, HB, 1, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, h1,
+                                                std::max(g, h0), s);
     }
-    cudaError_t e = launch_pass<WANT_G, HB, 0>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, 0, s);
+    used = g0 + g1;
+    cudaError_t e = launch_pass<WANT_G, HB, 0>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws, g0, 0, s);
     if (e != cudaSuccess) return e;
-    double* ws1 = ws ? ws + (size_t)vjp_grid(pl, 0, n) * m.R : nullptr;
-    return launch_pass<WANT_G, HB, 1>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws1, 0, s);
+    double* ws1 = ws ? ws + (size_t)g0 * m.R : nullptr;
+    return launch_pass<WANT_G, HB, 1>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, ws1, g1, 0, s);
 }
 
 }  // namespace
@@ -821,32 +829,36 @@ cudaError_t noalloc_scratch(void** ptr) {
 }
 
 
-size_t vjp_workspace_bytes(const DevMech& m, int64_t n) {
+// The workspace a call is given room for, or the least it does with.
+size_t vjp_workspace_bytes(const DevMech& m, int64_t n, bool least) {
     VjpPlan pl;
     if (!plan_for(m, true, false, pl)) return 0;
     VjpPlan pl2;
     if (!plan_for(m, true, true, pl2)) return 0;
-    const int64_t blocks = std::max(vjp_rows(pl, n), vjp_rows(pl2, n));   // either cotangent set
+    const int64_t blocks = least ? std::max(vjp_rows_least(pl, n), vjp_rows_least(pl2, n))
+                                 : std::max(vjp_rows(pl, n), vjp_rows(pl2, n));                // either cotangent set
     return (size_t)blocks * m.R * sizeof(double);
 }
 
 cudaError_t launch_vjp(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p, const double* Y,
                        const double* dlnA, const double* bar_omega, const double* bar_hrr, double* gT, double* gY,
-                       double* g_lnA, void* ws, cudaStream_t s) {
+                       double* g_lnA, void* ws, size_t ws_bytes, cudaStream_t s) {
     static_assert(kDfTabBytes <= kMathTabDoubles * sizeof(double), "table space");
     const bool want_g = g_lnA != nullptr, hb = bar_hrr != nullptr;
     VjpPlan pl;
     if (!plan_for(m, want_g, hb, pl)) return cudaErrorInvalidConfiguration;
     double* wsd = static_cast<double*>(ws);
+    const int64_t rows = want_g ? (int64_t)(ws_bytes / ((size_t)m.R * sizeof(double))) : (int64_t)1 << 40;
+    int64_t used = 0;
     cudaError_t e;
     if (want_g)
-        e = hb ? launch_v<true, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, wsd, s)
-               : launch_v<true, false>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, wsd, s);
+        e = hb ? launch_v<true, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, wsd, rows, used, s)
+               : launch_v<true, false>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, wsd, rows, used, s);
     else
-        e = hb ? launch_v<false, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, nullptr, s)
-               : launch_v<false, false>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, nullptr, s);
+        e = hb ? launch_v<false, true>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, nullptr, rows, used, s)
+               : launch_v<false, false>(pl, m, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, nullptr, rows, used, s);
     if (e != cudaSuccess || !want_g) return e;
-    reduce_blocks_kernel<<<(m.R + 31) / 32, 32 * kReduceWarps, 0, s>>>(wsd, (int)vjp_rows_used(pl, n), m.rxn, m.R, g_lnA);
+    reduce_blocks_kernel<<<(m.R + 31) / 32, 32 * kReduceWarps, 0, s>>>(wsd, (int)used, m.rxn, m.R, g_lnA);
     return cudaGetLastError();
 }
 

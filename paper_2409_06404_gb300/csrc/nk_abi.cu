@@ -1301,13 +1301,13 @@ nk_status nk_rates_vjp(const nk_mech* m, int64_t n, int64_t ld, const double* T,
     if (!bar_omega || !gT || !gY) return fail(NK_EINVAL, "bar_omega, gT and gY must not be NULL");
     if ((st = check_out({bar_omega, bar_hrr, gT, gY, g_lnA, dlnA, workspace})) != NK_OK) return st;
     if (g_lnA) {
-        const size_t need = nk::vjp_workspace_bytes(m->d, n);
+        const size_t need = nk::vjp_workspace_bytes(m->d, n, true);
         if (!workspace || workspace_bytes < need)
             return fail(NK_EINVAL, "g_lnA needs %zu bytes of workspace, got %zu", need,
                         workspace ? workspace_bytes : (size_t)0);
     }
     return launched(nk::launch_vjp(m->d, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, g_lnA, workspace,
-                                   (cudaStream_t)stream),
+                                   workspace_bytes, (cudaStream_t)stream),
                     "vjp kernel launch");
 }
 
@@ -1321,9 +1321,9 @@ nk_status nk_rates_vjp_noalloc(const nk_mech* m, int64_t n, int64_t ld, const do
     if (!bar_omega || !gT || !gY) return fail(NK_EINVAL, "bar_omega, gT and gY must not be NULL");
     if ((st = check_out({bar_omega, bar_hrr, gT, gY, g_lnA, dlnA})) != NK_OK) return st;
     void* scratch = nullptr;
+    const size_t cap = nk::kNoallocScratchDoubles * sizeof(double);
     if (g_lnA) {
-        const size_t need = nk::vjp_workspace_bytes(m->d, n);
-        const size_t cap = nk::kNoallocScratchDoubles * sizeof(double);
+        const size_t need = nk::vjp_workspace_bytes(m->d, n, true);
         if (need > cap)
             return fail(NK_EUNSUPPORTED,
                         "nk_rates_vjp_noalloc: the ln A partial sums need %zu bytes, more than its fixed %zu-byte "
@@ -1332,7 +1332,7 @@ nk_status nk_rates_vjp_noalloc(const nk_mech* m, int64_t n, int64_t ld, const do
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(no-allocation scratch)");
     }
     return launched(nk::launch_vjp(m->d, n, ld, T, p, Y, dlnA, bar_omega, bar_hrr, gT, gY, g_lnA, scratch,
-                                   (cudaStream_t)stream),
+                                   cap, (cudaStream_t)stream),
                     "vjp kernel launch");
 }
 

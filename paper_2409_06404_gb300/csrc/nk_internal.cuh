@@ -356,7 +356,7 @@ cudaError_t launch_jvp(const DevMech& m, int64_t n, int64_t ld, const double* T,
                        const double* Y, const double* dlnA, const double* vT, const double* vY,
                        double* omega, double* hrr, double* d_omega, double* d_hrr, cudaStream_t s,
                        int rhs = 0);
-size_t vjp_workspace_bytes(const DevMech& m, int64_t n);
+size_t vjp_workspace_bytes(const DevMech& m, int64_t n, bool least = false);
 size_t reactor_workspace_bytes(const DevMech& m, int64_t n, int krylov_dim, int precond, int linearized);
 cudaError_t reactor_step(const DevMech& m, int64_t n, double* T, const double* p, double* Y, double dt,
                          const nk_reactor_opts& o, nk_reactor_stats& st, void* ws, cudaStream_t s);
@@ -429,7 +429,7 @@ cudaError_t launch_jvp_linearized_compact(const DevMech& m, int64_t n, int64_t l
 cudaError_t launch_vjp(const DevMech& m, int64_t n, int64_t ld, const double* T, const double* p,
                        const double* Y, const double* dlnA, const double* bar_omega,
                        const double* bar_hrr, double* gT, double* gY, double* g_lnA,
-                       void* ws, cudaStream_t s);
+                       void* ws, size_t ws_bytes, cudaStream_t s);
 
 // Capacity of the fixed device scratch of nk_rates_vjp_noalloc (8 MiB of doubles).
 constexpr size_t kNoallocScratchDoubles = (size_t)1 << 20;
